@@ -618,7 +618,6 @@ struct tf_rows_state {
   int fp16;
   int nsm;
   uint16_t* w16;            // every product's weights, 16-bit, back to back
-  float* hws;               // the head's workspace, chunk x (P + 128 + Q) floats
   float* vec;               // the products' bias and gain vectors, each 16-byte aligned
   int doubling;             // fourier_scale[k + 3] == 2 fourier_scale[k] for every k
   int64_t chunk, cap;       // tracks per chunk; rows of the workspace (chunk * max_hits)
@@ -765,7 +764,6 @@ void tf_rows_destroy(trackfit_ctx* h) {
   tf_rows_state* r = h->rows;
   if (!r) return;
   tf_free(r->w16);
-  tf_free(r->hws);
   tf_free(r->vec);
   tf_free(r->row0);
   tf_free(r->tot);
@@ -836,7 +834,7 @@ int tf_rows_create(trackfit_ctx* h, const float* host_w) {
   const size_t xyw = attn ? D : (2 * H > D ? 2 * H : D);
   const size_t pw = attn ? 3 * D : 4 * H;
   const size_t row_bytes = 2 * (E + hsw + xyw + (attn ? D : 0)) + 4 * (pw + (attn ? 2 * D : 0));
-  const size_t track_bytes = (size_t)s.T * row_bytes + 4 * (2 * (size_t)s.P + s.Hh + s.Q) + 16;
+  const size_t track_bytes = (size_t)s.T * row_bytes + 4 * (size_t)s.P + 16;
   int64_t chunk = (int64_t)(RG_WS_BUDGET / track_bytes);
   if (chunk > 4194304) chunk = 4194304;
   chunk = chunk / PLAN_NT * PLAN_NT;
@@ -854,7 +852,6 @@ int tf_rows_create(trackfit_ctx* h, const float* host_w) {
   alloc((void**)&r->xy16, cap * xyw * 2);
   alloc((void**)&r->p32, cap * pw * 4);
   alloc((void**)&r->pooled, (size_t)chunk * s.P * 4);
-  alloc((void**)&r->hws, (size_t)chunk * (s.P + s.Hh + s.Q) * 4);
   if (attn) {
     alloc((void**)&r->o16, cap * D * 2);
     alloc((void**)&r->x32, cap * D * 4);
@@ -957,6 +954,7 @@ int tf_rows_create(trackfit_ctx* h, const float* host_w) {
       return TRACKFIT_ERR_UNSUPPORTED;
     }
   }
+  if (tf_head_prepare(s.P) != cudaSuccess) return TRACKFIT_ERR_CUDA;
   if (attn && (tf_attn::allow_smem<__half>(s.T, s.D, s.NH) != cudaSuccess ||
                tf_attn::allow_smem<__nv_bfloat16>(s.T, s.D, s.NH) != cudaSuccess))
     return TRACKFIT_ERR_CUDA;
@@ -1014,7 +1012,10 @@ int rows_chunk(trackfit_ctx* h, const float* hits, const int64_t* offs, const in
     dim3 grid((unsigned)nb, (unsigned)((s.D + 127) / 128));
     pool_mean_rows_kernel<<<grid, 128, 0, st>>>(r->x32, r->row0, nc, nb, s.T, s.D, r->pooled);
   }
-  return tf_simt_head_batched(s, h->off, h->d_w, r->pooled, nc, nb, r->hws, out, out_q, out_pool, err, st);
+  const cudaError_t e = tf_head(s, h->off, h->d_w, r->pooled, nc, nb, r->nsm, out, out_q, out_pool, err, st);
+  if (e == cudaSuccess) return TRACKFIT_OK;
+  tf_note_cuda(e, "head launch");
+  return TRACKFIT_ERR_CUDA;
 }
 
 }  // namespace

@@ -1,6 +1,6 @@
 // tcgen05 path: one persistent, warp-specialised kernel runs the whole encoder
 // forward (embedding, every minGRU layer, pooling) for the 16-bit-operand
-// configs; head_kernel then applies the regression head to the pooled vectors.
+// configs; the head (head.cu) then runs on the pooled vectors.
 //
 // Orientation: every per-hit matrix product is computed transposed,
 //   D[channel][hit] = W[channel][k] * Act[k][hit],
@@ -44,9 +44,8 @@ constexpr int NT = 608;                   // warp 0 TMA, warp 1 MMA issuer, warp
 constexpr int NE = 512;                   // epilogue threads
 constexpr int SEGW = 32;                  // hit columns per epilogue thread (half a slab)
 constexpr int TILE = 128;
-constexpr int SLAB = 64;
-constexpr int MAX_TRK_SLAB = 16;
-constexpr int MAX_TRK_TILE = 2 * MAX_TRK_SLAB;
+constexpr int SLAB = TF_SLAB;
+constexpr int MAX_TRK_TILE = 2 * TF_SLAB_TRACKS;
 constexpr int A_BLOCK = 128 * 64 * 2;     // one 128-row x 64-k 16-bit weight block
 constexpr int A_STAGE = 2 * A_BLOCK;      // a pipeline stage holds two consecutive blocks
 constexpr int MAX_SCHED = 2048;           // schedule entries per tile
@@ -54,8 +53,7 @@ constexpr int EB_BYTES = 160 * 256;       // Fourier operand: 160 k-rows x 128 h
 constexpr int MISC_BYTES = 10240;
 constexpr int SCHED_BYTES = 2 * MAX_SCHED * 4;   // both schedule tables, copied to shared memory
 constexpr int MAX_STAGES = 8;
-constexpr int SEG = 1024;                 // tracks per packing segment
-constexpr int64_t MAXB = 4194304;         // tracks per launch chunk
+constexpr int64_t MAXB = TF_PACK_TRACKS;  // tracks per launch chunk
 constexpr int64_t POOL_TRACKS = 1048576;  // tracks per launch chunk when the pooled means go to the internal buffer
 constexpr uint64_t WAIT_NS = 2000000000ull;   // bounded-wait limit (a handle's test hook may lower it)
 constexpr uint64_t DRAIN_NS = 200000000ull;
@@ -84,8 +82,8 @@ struct TcParams {
   float* out_q;
   float* pool;   // [B][D] pooled means (the caller's buffer or an internal one)
   float* xs;
-  const int32_t* slab_start;   // slab s = tracks order[slab_start[s] .. slab_start[s + 1])
-  const int32_t* order;        // tracks in packing order
+  const int2* slab;            // the packing (tf_pack): slab s = tracks order[slab[s].x ..], slab[s].y of them
+  const int32_t* order;
   const int32_t* n_slabs;
   const uint32_t* sched_p;   // per block: map | col/64 << 4 | row << 8
   const uint32_t* sched_m;   // per block: b offset | bsel << 13 | tcol/128 << 14 | S_* flags
@@ -673,8 +671,8 @@ __device__ __forceinline__ void load_tile(const TcParams& p, Misc* m, TileMeta* 
   for (int hf = 0; hf < 2; ++hf) {
     const int s = 2 * tile + hf;
     if (s >= n_slabs) break;
-    const int b0 = p.slab_start[s];
-    const int cnt = p.slab_start[s + 1] - b0;
+    const int2 sl = p.slab[s];
+    const int b0 = sl.x, cnt = sl.y;
     int n = 0, trk = 0;
     if (lane < cnt) {
       trk = p.order[b0 + lane];
@@ -1209,108 +1207,6 @@ __global__ void build_schedule(const __grid_constant__ TcParams p, uint32_t* sp,
   *count = n;
 }
 
-// ------------------------------------------------------------------ packing
-// Packing of one segment of up to SEG tracks into slabs of at most SLAB hits and
-// MAX_TRK_SLAB tracks (one warp per segment, decisions by lane 0 so the order is
-// deterministic): best fit over length buckets, each slab taking the longest
-// remaining track that still fits until none does; tracks with an invalid hit
-// count take a slot but no columns, at the end.  A track's results do not
-// depend on where it is packed.  Writes the segment's slice of the packing order
-// and the order positions where its slabs start.
-__global__ void __launch_bounds__(32) plan_pack(const int32_t* __restrict__ n_hits, int64_t B, int T,
-                                                int32_t* __restrict__ seg_count, int32_t* __restrict__ seg_slabs,
-                                                int32_t* __restrict__ order) {
-  __shared__ int32_t cnt[SLAB + 1], pos[SLAB + 2];
-  __shared__ int16_t len_of[SEG], items[SEG];
-  const int seg = blockIdx.x, lane = threadIdx.x;
-  const int64_t b0 = (int64_t)seg * SEG;
-  const int nt = (int)((b0 + SEG < B) ? SEG : B - b0);
-  for (int i = lane; i <= SLAB; i += 32) cnt[i] = 0;
-  __syncwarp();
-  for (int i = lane; i < nt; i += 32) {
-    int v = n_hits[b0 + i];
-    if (v < 1 || v > T) v = 0;
-    len_of[i] = (int16_t)v;
-  }
-  __syncwarp();
-  if (lane == 0) {
-    for (int i = 0; i < nt; ++i) ++cnt[len_of[i]];
-    pos[0] = 0;
-    for (int l = 0; l <= SLAB; ++l) pos[l + 1] = pos[l] + cnt[l];
-    for (int i = 0; i < nt; ++i) items[pos[len_of[i]]++] = (int16_t)i;   // pos[l] -> end of bucket l
-    int32_t* out = seg_slabs + (size_t)seg * (SEG + 1);
-    int o = 0, ns = 0, cap = SLAB, ntr = 0;
-    int remaining = nt - cnt[0];
-    out[ns++] = (int32_t)b0;
-    int top = T < SLAB ? T : SLAB;
-    while (remaining > 0) {
-      int l = cap < top ? cap : top;
-      while (l >= 1 && cnt[l] == 0) --l;
-      if (l >= 1 && ntr < MAX_TRK_SLAB) {
-        order[b0 + o++] = (int32_t)(b0 + items[pos[l] - cnt[l]]);   // bucket l, next in track order
-        --cnt[l];
-        cap -= l;
-        ++ntr;
-        --remaining;
-      } else {   // the slab is full: start the next one
-        out[ns++] = (int32_t)(b0 + o);
-        cap = SLAB;
-        ntr = 0;
-      }
-    }
-    for (int k = 0; k < cnt[0]; ++k) {   // invalid tracks
-      if (ntr == MAX_TRK_SLAB) {
-        out[ns++] = (int32_t)(b0 + o);
-        ntr = 0;
-      }
-      order[b0 + o++] = (int32_t)(b0 + items[pos[0] - cnt[0] + k]);
-      ++ntr;
-    }
-    if (o == 0) ns = 0;   // (an empty segment cannot occur: nt >= 1)
-    seg_count[seg] = ns;
-  }
-}
-
-// Exclusive scan of the per-segment slab counts (one block), total and sentinel.
-__global__ void plan_scan(const int32_t* __restrict__ seg_count, int nseg, int64_t B, int32_t* __restrict__ seg_off,
-                          int32_t* __restrict__ n_slabs, int32_t* __restrict__ slab_start) {
-  __shared__ int32_t part[1024];
-  const int tid = threadIdx.x;
-  const int per = (nseg + 1023) / 1024;
-  int32_t s = 0;
-  for (int i = 0; i < per; ++i) {
-    const int k = tid * per + i;
-    if (k < nseg) s += seg_count[k];
-  }
-  part[tid] = s;
-  __syncthreads();
-  for (int o = 1; o < 1024; o <<= 1) {
-    const int32_t v = tid >= o ? part[tid - o] : 0;
-    __syncthreads();
-    part[tid] += v;
-    __syncthreads();
-  }
-  int32_t run = part[tid] - s;
-  for (int i = 0; i < per; ++i) {
-    const int k = tid * per + i;
-    if (k < nseg) {
-      seg_off[k] = run;
-      run += seg_count[k];
-    }
-  }
-  if (tid == 1023) {
-    n_slabs[0] = part[1023];
-    slab_start[part[1023]] = (int32_t)B;
-  }
-}
-
-__global__ void plan_scatter(const int32_t* __restrict__ seg_count, const int32_t* __restrict__ seg_off,
-                             const int32_t* __restrict__ seg_slabs, int32_t* __restrict__ slab_start) {
-  const int seg = blockIdx.x;
-  const int cnt = seg_count[seg], off = seg_off[seg];
-  for (int i = threadIdx.x; i < cnt; i += blockDim.x) slab_start[off + i] = seg_slabs[(size_t)seg * (SEG + 1) + i];
-}
-
 // ------------------------------------------------------------------ UMMA probe
 // D[128][128] = A[128][K] * B[K][128] through the same TMA / descriptor / TMEM
 // path as the fused kernel (test hook for the operand layouts).
@@ -1434,150 +1330,6 @@ bool make_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, boo
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// ------------------------------------------------------------------ head
-// Pooled vector -> RMSNorm (gain g_h) -> W_h1 (D -> 128) + SiLU -> W_h2 (128 -> Q)
-// for every track, fp32 on the CUDA cores (the head of Sec. 3.2).  One CTA per SM
-// walks blocks of HEAD_TRK tracks with both weight matrices staged in shared
-// memory once per CTA; the fused kernel leaves the pooled means in global memory.
-struct HeadParams {
-  const float* pool;   // [B][D] pooled means
-  const int32_t* n_hits;
-  int64_t B;
-  int T, D, Q, NQ;
-  float rms_eps;
-  const float* g;     // [D]
-  const float* w1t;   // [D][128]
-  const float* b1;    // [128]
-  const float* w2;    // [Q][128]
-  const float* b2;    // [Q]
-  float* out;         // [B][5]
-  float* out_q;       // [B][Q] or null
-  float* out_pool;    // the caller's pooled buffer (invalid tracks -> NaN) or null
-  unsigned long long* err;
-};
-constexpr int HEAD_TRK = 32, HEAD_NT = 256;
-size_t head_smem_bytes(int D, int Q) {
-  return ((size_t)D * 128 + (size_t)Q * 128 + (size_t)HEAD_TRK * D + (size_t)HEAD_TRK * 128 + D + 128 + Q +
-          HEAD_TRK) * 4;
-}
-
-__global__ void __launch_bounds__(HEAD_NT, 1) head_kernel(const __grid_constant__ HeadParams hp) {
-  extern __shared__ float4 hsm4[];
-  const int D = hp.D, Q = hp.Q;
-  float* w1t = reinterpret_cast<float*>(hsm4);   // [D][128]
-  float* w2 = w1t + D * 128;                      // [Q][128]
-  float* xv = w2 + Q * 128;                       // [HEAD_TRK][D]
-  float* hid = xv + HEAD_TRK * D;                 // [HEAD_TRK][128]
-  float* gs = hid + HEAD_TRK * 128;               // [D]
-  float* b1s = gs + D;                            // [128]
-  float* b2s = b1s + 128;                         // [Q]
-  int* bad_s = reinterpret_cast<int*>(b2s + Q);   // [HEAD_TRK]
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  for (int i = tid; i < D * 32; i += HEAD_NT) reinterpret_cast<float4*>(w1t)[i] = reinterpret_cast<const float4*>(hp.w1t)[i];
-  for (int i = tid; i < Q * 32; i += HEAD_NT) reinterpret_cast<float4*>(w2)[i] = reinterpret_cast<const float4*>(hp.w2)[i];
-  for (int i = tid; i < D; i += HEAD_NT) gs[i] = hp.g[i];
-  for (int i = tid; i < 128; i += HEAD_NT) b1s[i] = hp.b1[i];
-  for (int i = tid; i < Q; i += HEAD_NT) b2s[i] = hp.b2[i];
-  __syncthreads();
-  const float qnan = __int_as_float(0x7fc00000);
-  const int64_t nblk = (hp.B + HEAD_TRK - 1) / HEAD_TRK;
-  for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
-    const int64_t t0 = blk * HEAD_TRK;
-    const int nt = (int)((hp.B - t0) < HEAD_TRK ? (hp.B - t0) : HEAD_TRK);
-    // RMSNorm of each pooled vector (one warp per track); padding rows and
-    // invalid tracks become zero rows whose outputs are replaced by NaN
-    for (int i = warp; i < HEAD_TRK; i += HEAD_NT / 32) {
-      float* row = xv + i * D;
-      bool bad = true;
-      if (i < nt) {
-        const int n = hp.n_hits[t0 + i];
-        bad = n < 1 || n > hp.T;
-      }
-      if (bad) {
-        for (int c = lane; c < D; c += 32) row[c] = 0.0f;
-        if (i < nt && hp.out_pool)
-          for (int c = lane; c < D; c += 32) hp.out_pool[(t0 + i) * D + c] = qnan;
-      } else {
-        const float4* src = reinterpret_cast<const float4*>(hp.pool + (t0 + i) * D);
-        float ss = 0.0f;
-        for (int c4 = lane; c4 < D / 4; c4 += 32) {
-          const float4 v = src[c4];
-          reinterpret_cast<float4*>(row)[c4] = v;
-          ss = fmaf(v.x, v.x, ss);
-          ss = fmaf(v.y, v.y, ss);
-          ss = fmaf(v.z, v.z, ss);
-          ss = fmaf(v.w, v.w, ss);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        const float r = 1.0f / sqrtf(ss / (float)D + hp.rms_eps);
-        for (int c = lane; c < D; c += 32) row[c] *= r * gs[c];
-      }
-      if (lane == 0) bad_s[i] = bad;
-    }
-    __syncthreads();
-    {   // hidden units 4*j4 .. 4*j4+3 of tracks 4*tg .. 4*tg+3 (16-byte loads of
-        // both operands: 8 loads per 64 FMAs); the sum over c runs in order
-      const int j4 = tid & 31, tg = tid >> 5;
-      float a[4][4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) a[r][u] = b1s[4 * j4 + u];
-#pragma unroll 2
-      for (int c = 0; c < D; c += 4) {
-        float4 w[4], xr[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) w[k] = *reinterpret_cast<const float4*>(w1t + (c + k) * 128 + 4 * j4);
-#pragma unroll
-        for (int r = 0; r < 4; ++r) xr[r] = *reinterpret_cast<const float4*>(xv + (4 * tg + r) * D + c);
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const float xk[4] = {xr[r].x, xr[r].y, xr[r].z, xr[r].w};
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            a[r][0] = fmaf(w[k].x, xk[k], a[r][0]);
-            a[r][1] = fmaf(w[k].y, xk[k], a[r][1]);
-            a[r][2] = fmaf(w[k].z, xk[k], a[r][2]);
-            a[r][3] = fmaf(w[k].w, xk[k], a[r][3]);
-          }
-        }
-      }
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-        *reinterpret_cast<float4*>(hid + (4 * tg + r) * 128 + 4 * j4) =
-            make_float4(silu(a[r][0]), silu(a[r][1]), silu(a[r][2]), silu(a[r][3]));
-    }
-    __syncthreads();
-    // outputs; the dot product for output o starts at column 4o (mod 128), so the
-    // rows of W_h2 read by one warp fall in different banks while the
-    // summation order stays a function of o alone (results do not depend on a
-    // track's position in the batch)
-    for (int idx = tid; idx < nt * Q; idx += HEAD_NT) {
-      const int i = idx / Q, o = idx - i * Q;
-      const float4* w = reinterpret_cast<const float4*>(w2 + o * 128);
-      const float4* hv = reinterpret_cast<const float4*>(hid + i * 128);
-      float acc = 0.0f;
-#pragma unroll 8
-      for (int u = 0; u < 32; ++u) {
-        const int j4 = (u + o) & 31;
-        const float4 a4 = w[j4], h4 = hv[j4];
-        acc = fmaf(a4.x, h4.x, acc);
-        acc = fmaf(a4.y, h4.y, acc);
-        acc = fmaf(a4.z, h4.z, acc);
-        acc = fmaf(a4.w, h4.w, acc);
-      }
-      acc += b2s[o];
-      const int64_t trk = t0 + i;
-      if (bad_s[i]) acc = qnan;
-      if (hp.out_q) hp.out_q[trk * Q + o] = acc;
-      if (o % hp.NQ == hp.NQ / 2) hp.out[trk * 5 + o / hp.NQ] = acc;
-    }
-    if (tid < nt && bad_s[tid]) atomicAdd(hp.err, 1ull);
-    __syncthreads();
-  }
-}
-
 }  // namespace
 
 struct tf_tc_state {
@@ -1588,15 +1340,13 @@ struct tf_tc_state {
   void* dev = nullptr;  // one allocation for all weights
   uint16_t *w_e1 = nullptr, *w_e2 = nullptr, *w_in = nullptr, *w_m = nullptr, *w_1 = nullptr, *w_2 = nullptr;
   float *b_e1 = nullptr, *b_e2 = nullptr, *g = nullptr, *b_in = nullptr, *b_m = nullptr, *b_1 = nullptr,
-        *b_2 = nullptr, *hg = nullptr, *hw1t = nullptr, *hb1 = nullptr, *hw2 = nullptr, *hb2 = nullptr;
-  int32_t *seg_count = nullptr, *seg_off = nullptr, *seg_slabs = nullptr, *slab_start = nullptr, *n_slabs = nullptr,
-          *order = nullptr;
+        *b_2 = nullptr;
+  void* pack = nullptr;   // packing buffers for MAXB tracks
   uint32_t* sched = nullptr;   // [2][MAX_SCHED]: producer entries, then MMA entries
   int n_sched = 0;
   float* xs = nullptr;
   uint8_t* fbuf = nullptr;
   float* pool = nullptr;   // pooled means when the caller passes no buffer [POOL_TRACKS][D]
-  size_t head_smem = 0;
   uint64_t wait_ns = WAIT_NS;   // test hook (trackfit_debug_wait_limit)
   int hold_tile = -1;
   CUtensorMap tm[NMAPS];
@@ -1656,7 +1406,7 @@ void tf_tc_destroy(trackfit_ctx* h) {
   if (!h || !h->tc) return;
   tf_tc_state* t = h->tc;
   tf_free(t->dev);
-  tf_free(t->seg_count);
+  tf_free(t->pack);
   tf_free(t->xs);
   tf_free(t->fbuf);
   tf_free(t->pool);
@@ -1691,15 +1441,13 @@ int tf_tc_create(trackfit_ctx* h, const float* W) {
   if (t->nst < 2) return TRACKFIT_ERR_UNSUPPORTED;
   t->off_misc = t->off_a + t->nst * A_STAGE;
   t->smem = (size_t)t->off_misc + MISC_BYTES + SCHED_BYTES + 1024;
-  t->head_smem = head_smem_bytes(D, s.Q);
-  if (t->head_smem > (size_t)smem_optin) return TRACKFIT_ERR_UNSUPPORTED;
 
   // ---- repack weights (bf16 GEMM operands, fp32 biases/head)
   const size_t n_e1 = (size_t)D * E, n_e2 = (size_t)D * D, n_in = (size_t)L * t->ROWS_IN * D,
                n_m = (size_t)L * D * t->KM, n_11 = (size_t)L * D * D;
   std::vector<uint16_t> we1(n_e1), we2(n_e2), win(n_in, 0), wm(n_m, 0), w1(n_11), w2(n_11);
   std::vector<float> bin((size_t)L * t->ROWS_IN, 0.0f), gg((size_t)L * D), bm((size_t)L * D), b1((size_t)L * D),
-      b2((size_t)L * D), hw1t((size_t)s.P * 128);
+      b2((size_t)L * D);
   uint16_t (*cv)(float) = fp16 ? fp16_bits : bf16_bits;
   for (size_t i = 0; i < n_e1; ++i) we1[i] = cv(W[o.emb_w1 + i]);
   for (size_t i = 0; i < n_e2; ++i) we2[i] = cv(W[o.emb_w2 + i]);
@@ -1738,8 +1486,6 @@ int tf_tc_create(trackfit_ctx* h, const float* W) {
       b2[(size_t)l * D + c] = W[lo.b2 + c];
     }
   }
-  for (int c = 0; c < s.P; ++c)
-    for (int j = 0; j < 128; ++j) hw1t[(size_t)c * 128 + j] = W[o.head_w1 + (size_t)j * s.P + c];
 
   // ---- one device allocation for everything the kernel reads
   struct Part {
@@ -1761,11 +1507,6 @@ int tf_tc_create(trackfit_ctx* h, const float* W) {
       {bm.data(), bm.size() * 4, (void**)&t->b_m},
       {b1.data(), b1.size() * 4, (void**)&t->b_1},
       {b2.data(), b2.size() * 4, (void**)&t->b_2},
-      {W + o.head_g, (size_t)s.P * 4, (void**)&t->hg},
-      {hw1t.data(), hw1t.size() * 4, (void**)&t->hw1t},
-      {W + o.head_b1, (size_t)128 * 4, (void**)&t->hb1},
-      {W + o.head_w2, (size_t)s.Q * 128 * 4, (void**)&t->hw2},
-      {W + o.head_b2, (size_t)s.Q * 4, (void**)&t->hb2},
   };
   size_t total = 0;
   for (auto& pt : parts) total += (pt.bytes + 255) & ~(size_t)255;
@@ -1777,14 +1518,7 @@ int tf_tc_create(trackfit_ctx* h, const float* W) {
     off += (pt.bytes + 255) & ~(size_t)255;
   }
   // ---- packing buffers and the per-CTA residual scratch
-  const int nseg_max = (int)((MAXB + SEG - 1) / SEG);
-  const size_t plan_ints = (size_t)nseg_max * 2 + (size_t)nseg_max * (SEG + 1) + (size_t)MAXB + 2 + 64 + (size_t)MAXB;
-  if (tf_malloc((void**)&t->seg_count, plan_ints * 4) != cudaSuccess) return TRACKFIT_ERR_OOM;
-  t->seg_off = t->seg_count + nseg_max;
-  t->seg_slabs = t->seg_off + nseg_max;
-  t->slab_start = t->seg_slabs + (size_t)nseg_max * (SEG + 1);
-  t->n_slabs = t->slab_start + MAXB + 2;
-  t->order = t->n_slabs + 64;
+  if (tf_malloc(&t->pack, tf_pack_bytes(MAXB)) != cudaSuccess) return TRACKFIT_ERR_OOM;
   if (tf_malloc((void**)&t->xs, (size_t)t->nsm * TILE * D * sizeof(float)) != cudaSuccess) return TRACKFIT_ERR_OOM;
   if (tf_malloc((void**)&t->fbuf, (size_t)t->nsm * 2 * EB_BYTES) != cudaSuccess) return TRACKFIT_ERR_OOM;
   if (tf_malloc((void**)&t->pool, (size_t)POOL_TRACKS * D * sizeof(float)) != cudaSuccess) return TRACKFIT_ERR_OOM;
@@ -1814,8 +1548,7 @@ int tf_tc_create(trackfit_ctx* h, const float* W) {
           cudaSuccess ||
       cudaFuncSetAttribute(tc_forward_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t->smem) !=
           cudaSuccess ||
-      cudaFuncSetAttribute(head_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t->head_smem) !=
-          cudaSuccess)
+      tf_head_prepare(s.P) != cudaSuccess)
     return TRACKFIT_ERR_CUDA;
   return TRACKFIT_OK;
 }
@@ -1829,9 +1562,10 @@ int tf_tc_forward(trackfit_ctx* h, const float* hits, const int32_t* n_hits, int
   for (int i = 0; i < NMAPS; ++i) p.tm[i] = t->tm[i];
   p.xs = t->xs;
   p.fbuf = t->fbuf;
-  p.slab_start = t->slab_start;
-  p.order = t->order;
-  p.n_slabs = t->n_slabs;
+  const tf_pack pk = tf_pack_in(t->pack, MAXB);
+  p.slab = pk.slab;
+  p.order = pk.order;
+  p.n_slabs = pk.n_slabs;
   p.sched_p = t->sched;
   p.sched_m = t->sched + MAX_SCHED;
   p.n_sched = t->n_sched;
@@ -1871,28 +1605,12 @@ int tf_tc_forward(trackfit_ctx* h, const float* hits, const int32_t* n_hits, int
   p.scale_doubling = 1;
   for (int k = 0; k + 3 < 16; ++k)
     if (s.scale[k + 3] != 2.0f * s.scale[k]) p.scale_doubling = 0;
-  HeadParams hp;
-  std::memset(&hp, 0, sizeof(hp));
-  hp.T = s.T;
-  hp.D = s.D;
-  hp.Q = s.Q;
-  hp.NQ = s.NQ;
-  hp.rms_eps = s.rms_eps;
-  hp.g = t->hg;
-  hp.w1t = t->hw1t;
-  hp.b1 = t->hb1;
-  hp.w2 = t->hw2;
-  hp.b2 = t->hb2;
-  hp.err = h->d_err;
   // without a caller buffer the pooled means go to the internal one, which
   // bounds the launch chunk
   const int64_t chunk = out_pool ? MAXB : POOL_TRACKS;
   for (int64_t c0 = 0; c0 < B; c0 += chunk) {
     const int64_t nb = (B - c0 < chunk) ? B - c0 : chunk;
-    const int nseg = (int)((nb + SEG - 1) / SEG);
-    plan_pack<<<nseg, 32, 0, st>>>(n_hits + c0, nb, s.T, t->seg_count, t->seg_slabs, t->order);
-    plan_scan<<<1, 1024, 0, st>>>(t->seg_count, nseg, nb, t->seg_off, t->n_slabs, t->slab_start);
-    plan_scatter<<<nseg, 128, 0, st>>>(t->seg_count, t->seg_off, t->seg_slabs, t->slab_start);
+    if (tf_plan(n_hits + c0, nb, s.T, t->nsm, pk.order, pk.slab, pk.n_slabs, st) != cudaSuccess) return TRACKFIT_ERR_CUDA;
     p.hits = offs ? hits : hits + c0 * s.T * 5;
     p.offs = offs ? offs + c0 : nullptr;
     p.n_hits = n_hits + c0;
@@ -1905,13 +1623,9 @@ int tf_tc_forward(trackfit_ctx* h, const float* hits, const int32_t* n_hits, int
     else
       tc_forward_kernel<false><<<t->nsm, NT, t->smem, st>>>(p);
     tf_prof_end(h, st);
-    hp.pool = p.pool;
-    hp.n_hits = p.n_hits;
-    hp.B = nb;
-    hp.out = p.out;
-    hp.out_q = p.out_q;
-    hp.out_pool = out_pool ? p.pool : nullptr;
-    head_kernel<<<t->nsm, HEAD_NT, t->head_smem, st>>>(hp);
+    if (tf_head(s, h->off, h->d_w, p.pool, p.n_hits, nb, t->nsm, p.out, p.out_q, out_pool ? p.pool : nullptr, h->d_err,
+                st) != cudaSuccess)
+      return TRACKFIT_ERR_CUDA;
     if (cudaPeekAtLastError() != cudaSuccess) return TRACKFIT_ERR_CUDA;
   }
   return TRACKFIT_OK;

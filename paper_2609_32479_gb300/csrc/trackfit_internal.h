@@ -20,6 +20,9 @@ struct tf_nvtx_range {
 
 #define TF_MAX_LAYERS 16
 #define TF_MAX_HITS 64
+#define TF_SLAB 64          // hits of a slab of packed tracks
+#define TF_SLAB_TRACKS 16   // tracks of a slab
+#define TF_PACK_TRACKS 4194304  // tracks that a handle packs at a time
 #define TF_PACKED_CHUNK 1048576
 #define TF_HOST_CHUNK 262144  // tracks per copy / compute step of trackfit_forward_host
 #define TF_HOST_EVENTS 10
@@ -93,14 +96,32 @@ int tf_simt_workspace(trackfit_ctx* h);
 // offs (may be null): packed input, track b's hits are rows offs[b] .. of hits
 int tf_simt_forward(trackfit_ctx* h, const float* hits, const int32_t* n_hits, int64_t B,
                     float* out, float* out_q, float* out_pool, cudaStream_t st, const int64_t* offs = nullptr);
-int tf_simt_head(const tf_shape& s, const tf_blob_off& o, const float* W, const float* pooled,
-                 const int32_t* n_hits, int64_t B, float* out, float* out_q, float* out_pool,
-                 unsigned long long* err, cudaStream_t st);
-int tf_simt_head_batched(const tf_shape& s, const tf_blob_off& o, const float* W, const float* pooled,
-                         const int32_t* n_hits, int64_t B, float* ws, float* out, float* out_q, float* out_pool,
-                         unsigned long long* err, cudaStream_t st);
 int tf_simt_debug_scan(const float* a, const float* b, const float* x, const int32_t* n_hits,
                        int64_t B, int T, int C, float* hf, float* hb, cudaStream_t st);
+
+// plan.cu: tracks packed whole into slabs.  Slab i holds the tracks order[slab[i].x]
+// .. order[slab[i].x + slab[i].y - 1]; n_slabs[0] slabs for up to cap tracks.
+struct tf_pack {
+  int32_t* order;
+  int2* slab;
+  int32_t* n_slabs;
+  int64_t cap;
+};
+cudaError_t tf_plan(const int32_t* n_hits, int64_t B, int T, int nsm, int32_t* order, int2* slab, int32_t* n_slabs,
+                    cudaStream_t st);
+// The three arrays of tf_pack in one buffer of tf_pack_bytes(cap) bytes.
+inline size_t tf_pack_bytes(int64_t cap) { return 256 + (size_t)cap * 12; }
+inline tf_pack tf_pack_in(void* buf, int64_t cap) {
+  char* b = static_cast<char*>(buf);
+  return {reinterpret_cast<int32_t*>(b + 256 + cap * 8), reinterpret_cast<int2*>(b + 256),
+          reinterpret_cast<int32_t*>(b), cap};
+}
+
+// head.cu
+cudaError_t tf_head_prepare(int P);   // shared memory of the launches below
+cudaError_t tf_head(const tf_shape& s, const tf_blob_off& o, const float* W, const float* pooled,
+                    const int32_t* n_hits, int64_t B, int nsm, float* out, float* out_q, float* out_pool,
+                    unsigned long long* err, cudaStream_t st);
 
 // tc_forward.cu
 bool tf_tc_supported(const tf_shape& s);
