@@ -242,6 +242,7 @@ extern "C" void trackfit_destroy(trackfit_t h) {
   tf_free(h->d_w);
   tf_free(h->d_err);
   tf_free(h->ws);
+  tf_free(h->pack);
   tf_free(h->pk_n);
   tf_free(h->st_hits);
   tf_free(h->st_n);

@@ -54,9 +54,10 @@ extern "C" int trackfit_forward_noalloc(const trackfit_config_t* cfg, const floa
                         reinterpret_cast<uintptr_t>(n_hits) | reinterpret_cast<uintptr_t>(weights);
   if (mis & 15u) return TRACKFIT_ERR_INVALID_ARG;
   const size_t counter_bytes = 256;
+  const bool fused = tf_fused_fp32_supported(s);   // needs only the packing's buffers
   const size_t per_track = tf_simt_bytes_per_track(s);
   const int64_t fit = (int64_t)((TF_NOALLOC_SCRATCH_BYTES - counter_bytes) / per_track);
-  if (fit < 1) return TRACKFIT_ERR_UNSUPPORTED;   // one track's workspace exceeds the array
+  if (!fused && fit < 1) return TRACKFIT_ERR_UNSUPPORTED;   // one track's workspace exceeds the array
   int64_t chunk = fit;
   if (chunk > 65535) chunk = 65535;
   if (chunk * s.T > 65535LL * 64) chunk = 65535LL * 64 / s.T;
@@ -68,6 +69,12 @@ extern "C" int trackfit_forward_noalloc(const trackfit_config_t* cfg, const floa
                                                                   TF_NOALLOC_SCRATCH_BYTES - counter_bytes);
   // the array keeps the previous call's contents: the counter must start at zero
   if (cudaMemsetAsync(err, 0, sizeof(unsigned long long), cs) != cudaSuccess) return TRACKFIT_ERR_CUDA;
+  if (fused) {
+    if (tf_fused_fp32_prepare(s) != cudaSuccess) return TRACKFIT_ERR_CUDA;
+    const int64_t cap = (int64_t)((TF_NOALLOC_SCRATCH_BYTES - counter_bytes - tf_pack_bytes(0)) / 12);
+    return tf_fused_fp32_forward(s, o, weights, tf_pack_in(base, cap), err, hits, n_hits, nullptr, n_tracks, out_params,
+                                 nullptr, nullptr, cs, nullptr);
+  }
   return tf_simt_forward_explicit(s, o, weights, static_cast<float*>(base), chunk, err, hits, n_hits, n_tracks,
                                   out_params, cs);
 }

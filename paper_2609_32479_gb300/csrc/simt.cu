@@ -1,5 +1,6 @@
-// SIMT (CUDA-core) kernel path: the production path for TRACKFIT_FP32 configs
-// and a second, independent GPU implementation of the BF16_PROJ arithmetic.
+// SIMT (CUDA-core) kernel path, a launch a step: the TRACKFIT_FP32 configs that the
+// fused fp32 encoder (fused_fp32.cu) does not take, and a second, independent GPU
+// implementation of the BF16_PROJ arithmetic.
 //
 // Layout: the batch is processed in chunks of whole tracks; inside a chunk every
 // per-hit tensor is row-major [tracks * max_hits][channels] in the handle's
@@ -287,7 +288,12 @@ int launch_gemm(const GemmArgs& g, cudaStream_t st) {
 
 }  // namespace
 
+// fp32 handles that the fused encoder takes need only the packing's buffers.
 int tf_simt_workspace(trackfit_ctx* h) {
+  if (tf_fused_fp32_supported(h->s)) {
+    const int e = tf_status_from_cuda(tf_malloc(&h->pack, tf_pack_bytes(TF_PACK_TRACKS)));
+    return e != TRACKFIT_OK ? e : tf_status_from_cuda(tf_fused_fp32_prepare(h->s));
+  }
   const size_t budget = (size_t)1 << 30;
   size_t per = ws_floats_per_track(h->s) * sizeof(float);
   int64_t n = (int64_t)(budget / per);
@@ -407,6 +413,9 @@ int tf_simt_run(const tf_shape& s, const tf_blob_off& o, const float* W, float* 
 
 int tf_simt_forward(trackfit_ctx* h, const float* hits, const int32_t* n_hits, int64_t B, float* out,
                     float* out_q, float* out_pool, cudaStream_t st, const int64_t* offs) {
+  if (h->pack)
+    return tf_fused_fp32_forward(h->s, h->off, h->d_w, tf_pack_in(h->pack, TF_PACK_TRACKS), h->d_err, hits, n_hits,
+                                 offs, B, out, out_q, out_pool, st, h);
   return tf_simt_run(h->s, h->off, h->d_w, h->ws, h->ws_tracks, h->d_err, hits, n_hits, B, out, out_q, out_pool, st,
                      h, offs);
 }

@@ -66,6 +66,7 @@ struct trackfit_ctx {
   float* ws;
   size_t ws_bytes;
   int64_t ws_tracks;
+  void* pack;                    // fused fp32 encoder: packing buffers for TF_PACK_TRACKS tracks
   // packed input: per-track hit counts derived from the offsets, one chunk of
   // TF_PACKED_CHUNK tracks at a time
   int32_t* pk_n;
@@ -122,6 +123,13 @@ cudaError_t tf_head_prepare(int P);   // shared memory of the launches below
 cudaError_t tf_head(const tf_shape& s, const tf_blob_off& o, const float* W, const float* pooled,
                     const int32_t* n_hits, int64_t B, int nsm, float* out, float* out_q, float* out_pool,
                     unsigned long long* err, cudaStream_t st);
+
+// fused_fp32.cu
+bool tf_fused_fp32_supported(const tf_shape& s);
+cudaError_t tf_fused_fp32_prepare(const tf_shape& s);
+int tf_fused_fp32_forward(const tf_shape& s, const tf_blob_off& o, const float* W, const tf_pack& pk,
+                          unsigned long long* err, const float* hits, const int32_t* n_hits, const int64_t* offs,
+                          int64_t B, float* out, float* out_q, float* out_pool, cudaStream_t st, trackfit_ctx* prof);
 
 // tc_forward.cu
 bool tf_tc_supported(const tf_shape& s);

@@ -1,5 +1,6 @@
-"""Sizes where a kernel's split can go wrong, against the oracle: the head's two CTA
-sizes, and the seed's foot points on strongly curved tracks."""
+"""Sizes where a kernel's split can go wrong, against the oracle: the fused fp32
+encoder (each column tiling, 16- and 64-row CTAs, runs of tracks and packed slabs),
+the head's two CTA sizes, and the seed's foot points on strongly curved tracks."""
 import dataclasses
 
 import numpy as np
@@ -8,7 +9,7 @@ import pytest
 from oracle import seed_oracle as S
 from oracle import trackfit_oracle as O
 from paper_2609_32479_gb300 import workloads as W
-from tests.helpers import FP16_TOL, track_errors
+from tests.helpers import FP16_TOL, FP32_TOL, track_errors
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -33,6 +34,33 @@ def forward(T, model, blob, hits, n_hits):
         tf.forward(h, n, out)
         torch.cuda.synchronize()
         return out.cpu().numpy(), tf.device_errors()
+
+
+def ragged(model, n, seed=3):
+    w = W.Workload("t", n, model, layout="sweep", n_barrel=model.max_hits, min_hits=model.max_hits)
+    n_hits = np.random.default_rng(seed).integers(1, model.max_hits + 1, n).astype(np.int32)
+    return W.gen_tracks(w, seed=seed).hits, n_hits
+
+
+# (d_model, max_hits, tracks, pool): every pair of column tilings; 16-row CTAs (a
+# track or two each), 64-row CTAs of consecutive tracks, packed slabs (more tracks than
+# the CTA slots take at once), a one-track batch, slabs full of one- and 64-hit tracks
+@pytest.mark.parametrize("D,hits,n,pool", [
+    (16, 5, 1, 0), (32, 10, 305, 0), (32, 16, 304, 1), (48, 9, 911, 0), (64, 12, 1530, 0), (64, 64, 40, 1),
+    (80, 17, 70, 0), (96, 24, 700, 1), (112, 8, 33, 0), (128, 24, 153, 0), (128, 3, 2500, 1)])
+def test_fused_fp32_encoder_shapes(T, D, hits, n, pool):
+    m = W.ModelConfig(max_hits=hits, d_model=D, d_hidden=3 * D // 2, n_layers=2, pool=pool)
+    blob = W.gen_weights(m, 2)
+    h, nh = ragged(m, n)
+    bad = n // 2 if n > 8 else None
+    if bad:
+        nh[bad] = hits + 1
+    got, (status, n_bad) = forward(T, m, blob, h, nh)
+    ref = O.forward(dataclasses.asdict(m), blob, h, nh)
+    ok = ~np.isnan(ref[:, 0])
+    assert n_bad == (1 if bad else 0) and status == (T.ERR_BAD_HITS if bad else T.OK)
+    np.testing.assert_array_equal(np.isnan(got), np.isnan(ref))
+    assert track_errors(got[ok], ref[ok]).max() <= FP32_TOL
 
 
 @pytest.mark.parametrize("n", [1, 16, 17, 4865])
