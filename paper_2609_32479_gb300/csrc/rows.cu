@@ -615,6 +615,7 @@ __global__ void pool_mean_rows_kernel(const float* __restrict__ x, const int64_t
 
 // ------------------------------------------------------------------ host side
 struct tf_rows_state {
+  tf_cat_state* cat;        // the configurations that concat.cu takes: nothing below but wait_ns is set up then
   int fp16;
   int nsm;
   uint16_t* w16;            // every product's weights, 16-bit, back to back
@@ -763,6 +764,7 @@ bool tf_rows_supported(const tf_shape& s) {
 void tf_rows_destroy(trackfit_ctx* h) {
   tf_rows_state* r = h->rows;
   if (!r) return;
+  tf_cat_destroy(r->cat);
   tf_free(r->w16);
   tf_free(r->vec);
   tf_free(r->row0);
@@ -793,6 +795,7 @@ int tf_rows_create(trackfit_ctx* h, const float* host_w) {
   h->rows = r;   // freed by tf_rows_destroy on any failure below
   r->fp16 = s.precision == TRACKFIT_FP16_PROJ;
   r->wait_ns = RG_WAIT_NS;
+  if (tf_cat_supported(s)) return tf_cat_create(h, host_w, &r->cat);
   r->doubling = 1;
   for (int k = 0; k + 3 < TRACKFIT_MAX_FOURIER; ++k)
     if (s.scale[k + 3] != 2.0f * s.scale[k]) r->doubling = 0;
@@ -1024,6 +1027,7 @@ int tf_rows_forward(trackfit_ctx* h, const float* hits, const int32_t* n_hits, i
                     float* out_q, float* out_pool, cudaStream_t st, const int64_t* offs) {
   tf_rows_state* r = h->rows;
   const tf_shape& s = h->s;
+  if (r->cat) return tf_cat_forward(h, r->cat, r->wait_ns, hits, n_hits, B, out, out_q, out_pool, st, offs);
   for (int64_t c0 = 0; c0 < B; c0 += r->chunk) {
     const int64_t nb = B - c0 < r->chunk ? B - c0 : r->chunk;
     const float* hc = offs ? hits : hits + c0 * s.T * s.F;

@@ -430,8 +430,10 @@ __device__ __forceinline__ void scan_gates(const ECtx& x, float (&z)[32], float 
 // finite state coming from the padding is multiplied away).  Values left in
 // padding columns stay in padding columns (every product and norm is per
 // column) and stay finite (their x_hat is 0), so they need no clearing here.
-template <bool FP16>
-__device__ __forceinline__ void scan_chain_store(const ECtx& x, float (&a)[32], const float (&b)[32]) {
+// SELECT: the state after a restart is b itself, so that an infinity or NaN of one
+// track stays out of the next (a second, predicated instruction on the serial path).
+template <bool SELECT>
+__device__ __forceinline__ void scan_chain(const ECtx& x, float (&a)[32], const float (&b)[32]) {
   const bool fwd = x.q < 2;
   const bool leads = fwd ? x.sub == 0 : x.sub == 1;
   float h = 0.0f;
@@ -439,23 +441,33 @@ __device__ __forceinline__ void scan_chain_store(const ECtx& x, float (&a)[32], 
     carry_wait(x);
     h = x.carry[x.half][x.c];
   }
+  const uint32_t rm = fwd ? x.md->m_first[x.half][x.sub] : x.md->m_last[x.half][x.sub];
+  auto step = [&](int j) {
+    if constexpr (SELECT) {
+      asm("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\t"
+          "@!p fma.rn.f32 %0, %1, %0, %2;\n\t@p mov.f32 %0, %2;\n\t}"
+          : "+f"(h)
+          : "f"(a[j]), "f"(b[j]), "r"(rm & (1u << j)));
+    } else {
+      h = fmaf(a[j], h, b[j]);
+    }
+    a[j] = h;
+  };
   if (fwd) {
 #pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      h = fmaf(a[j], h, b[j]);
-      a[j] = h;
-    }
+    for (int j = 0; j < 32; ++j) step(j);
   } else {
 #pragma unroll
-    for (int j = 31; j >= 0; --j) {
-      h = fmaf(a[j], h, b[j]);
-      a[j] = h;
-    }
+    for (int j = 31; j >= 0; --j) step(j);
   }
   if (leads) {
     x.carry[x.half][x.c] = h;
     carry_pass(x);
   }
+}
+template <bool FP16>
+__device__ __forceinline__ void scan_chain_store(const ECtx& x, float (&a)[32], const float (&b)[32]) {
+  scan_chain<false>(x, a, b);
   store_row32<FP16>(x.hb, x.c, x.col0, a);
 }
 
@@ -464,9 +476,8 @@ __device__ __forceinline__ void scan_chain_store(const ECtx& x, float (&a)[32], 
 // the metadata buffer md), the features of its hits, and the Fourier operand
 // (the B operand of the embedding's first product) as the byte image of HB in
 // the CTA's global buffer fb, from which the epilogue copies it at tile start.
-template <bool FP16>
-__device__ __forceinline__ void load_tile(const TileSrc& p, LoaderScratch* m, TileMeta* md, uint8_t* fb, int tile,
-                                          int n_slabs, int lane) {
+__device__ __forceinline__ void load_meta(const TileSrc& p, uint8_t* col_tpos, TileMeta* md, int tile, int n_slabs,
+                                          int lane) {
   for (int c = lane; c < TILE; c += 32) md->col_flags[c] = 0;
   __syncwarp();
   int ns = 0;
@@ -496,7 +507,7 @@ __device__ __forceinline__ void load_tile(const TileSrc& p, LoaderScratch* m, Ti
         const int col = c0 + t;
         md->col_flags[col] = (uint8_t)(F_VALID | (t == 0 ? F_FIRST : 0) | (t == n - 1 ? F_LAST : 0));
         md->col_slot[col] = (uint8_t)slot;
-        m->col_tpos[col] = (uint8_t)t;
+        if (col_tpos) col_tpos[col] = (uint8_t)t;
       }
     }
     ns += cnt;
@@ -515,6 +526,13 @@ __device__ __forceinline__ void load_tile(const TileSrc& p, LoaderScratch* m, Ti
     md->m_last[hf][w] = lm;
     md->m_valid[hf][w] = vm;
   }
+  __syncwarp();
+}
+
+template <bool FP16>
+__device__ __forceinline__ void load_tile(const TileSrc& p, LoaderScratch* m, TileMeta* md, uint8_t* fb, int tile,
+                                          int n_slabs, int lane) {
+  load_meta(p, m->col_tpos, md, tile, n_slabs, lane);
   for (int idx = lane; idx < TILE * 5; idx += 32) {
     const int col = idx / 5, f = idx - col * 5;
     float v = 0.0f;

@@ -142,6 +142,14 @@ int tf_tc_forward(trackfit_ctx* h, const float* hits, const int32_t* n_hits, int
 int tf_tc_wait_limit(trackfit_ctx* h, int64_t limit_ns, int hold_tile);
 int tf_tc_probe(trackfit_ctx* h, const uint16_t* A, const uint16_t* Bkn, int K, float* D, cudaStream_t st);
 
+// concat.cu: the paper's model in one kernel, behind the handle of rows.cu
+struct tf_cat_state;
+bool tf_cat_supported(const tf_shape& s);
+int tf_cat_create(trackfit_ctx* h, const float* host_w, tf_cat_state** out);
+void tf_cat_destroy(tf_cat_state* c);
+int tf_cat_forward(trackfit_ctx* h, tf_cat_state* c, uint64_t wait_ns, const float* hits, const int32_t* n_hits,
+                   int64_t B, float* out, float* out_q, float* out_pool, cudaStream_t st, const int64_t* offs);
+
 // rows.cu
 bool tf_rows_supported(const tf_shape& s);
 int tf_rows_create(trackfit_ctx* h, const float* host_w);
