@@ -72,21 +72,52 @@ __device__ __forceinline__ float silu(float x) { return x * sigm(x); }
 // oracle).  The output gate does not: its value scales the merge into the fp32
 // residual stream, where that error showed up on every track, so it takes the
 // two-operation sigmoid, as do the scan gates (a = 1 - sigma there also needs
-// relative accuracy as sigma -> 1).  (A reciprocal by Newton steps on the FMA
-// pipe instead of rcp was measured slower: these epilogues are bound by issued
-// instructions more than by the MUFU unit.)  sigm_pre takes its argument
-// already scaled by -log2 e, with the bias folded in by one FMA.
-__device__ __forceinline__ float sigm_pre(float t) { return rcp_approx(1.0f + ex2_approx(t)); }
+// relative accuracy as sigma -> 1).
 __device__ __forceinline__ float tanh_approx(float x) {
   float y;
   asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// SiLU(v + b) in that form, with hb = b / 2: the half argument (v + b) / 2 comes
-// from one FMA, bit for bit the value of halving the rounded sum (halving is exact)
-__device__ __forceinline__ float silu_tb(float v, float hb) {
-  const float h = fmaf(v, 0.5f, hb);
-  return fmaf(h, tanh_approx(h), h);
+// Two floats in one 64-bit register: the packed fp32 operations are the IEEE ones on each
+// half and take one issue slot for two values.
+struct f2 {
+  uint64_t v;
+  __device__ __forceinline__ f2(float a, float b) { asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b)); }
+  __device__ __forceinline__ explicit f2(float a) : f2(a, a) {}
+  __device__ __forceinline__ void get(float& a, float& b) const { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+};
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(a.v) : "l"(a.v), "l"(b.v));
+  return a;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(a.v) : "l"(a.v), "l"(b.v));
+  return a;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(a.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return a;
+}
+// For two arguments t = -x log2 e: e = 2^t and sigma(x) = 1 / (1 + e).  The
+// special-function unit bounds the gates (16 results a cycle and SM; with ex2 and rcp they
+// took 1.9 k cycles a chunk of 512 threads x 32), so the reciprocal is formed on the
+// multiply-add pipe, two at a time: the exponent-negating integer subtraction (0.0505
+// off at most, the least of any constant), a step of third order and a Newton step leave
+// 7.6e-8 at most over [1, 2^60], as the hardware's.  t is held at 60, which keeps that range: sigma is then 8.7e-19 instead
+// of less.  (One rcp for a pair of values would make a hit's result depend on its
+// neighbour's.)
+__device__ __forceinline__ void sigmoid2(f2 t, f2& e, f2& sg) {
+  float t0, t1, d0, d1;
+  t.get(t0, t1);
+  e = f2(ex2_approx(fminf(t0, 60.0f)), ex2_approx(fminf(t1, 60.0f)));
+  f2 d = add2(e, f2(1.0f));
+  d.get(d0, d1);
+  const f2 y(__uint_as_float(0x7ef311c0u - __float_as_uint(d0)), __uint_as_float(0x7ef311c0u - __float_as_uint(d1)));
+  d = f2(-d0, -d1);
+  f2 r = fma2(d, y, f2(1.0f));
+  sg = fma2(y, fma2(r, r, r), y);
+  r = fma2(d, sg, f2(1.0f));
+  sg = fma2(sg, r, sg);
 }
 
 // Operand conversion (round to nearest even): bf16, or fp16 when FP16 is set.
@@ -172,15 +203,22 @@ __device__ __forceinline__ void carry_wait(const ECtx& x) {
   asm volatile("bar.sync %0, 64;" ::"r"(2 + 2 * x.q + x.half) : "memory");
 }
 
-// silu(acc + b) of the 128-channel tile mt -> k-rows row0 + c of buf (b: the
+// silu(acc + b) of the 128-channel tile mt, with the half argument from one FMA (the
+// rounded sum halved: exact) -> k-rows row0 + c of buf (b: the
 // thread's channel's bias, loaded before the wait for the product)
 template <bool FP16>
 __device__ __forceinline__ void ep_silu_mt(const ECtx& x, float b, int mt, uint32_t buf, int row0) {
   float v[32];
   tmem_ld32(x.gt + mt * 128 + x.col0, v);
   tmem_ld_wait();
+  const f2 hb(0.5f * b);
 #pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = silu_tb(v[i], 0.5f * b);
+  for (int i = 0; i < 32; i += 2) {
+    const f2 h = fma2(f2(v[i], v[i + 1]), f2(0.5f), hb);
+    float h0, h1;
+    h.get(h0, h1);
+    fma2(h, f2(tanh_approx(h0), tanh_approx(h1)), h).get(v[i], v[i + 1]);
+  }
   store_row32<FP16>(buf, row0 + x.c, x.col0, v);
 }
 // silu(acc + bias) of the embedding's first product (in the gate columns) -> XB rows [mt*128 + c], all tiles read under one TMEM wait;
@@ -261,9 +299,9 @@ __device__ __forceinline__ void ep_residual(const ECtx& x, const float* bias, co
       tmem_ld16(x.acc + mt * 128 + x.col0 + 16 * hh, v);
       tmem_ld_wait();
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const float val = v[i] + bias_v[mt];
-        sq[16 * hh + i] = fmaf(val, val, sq[16 * hh + i]);
+      for (int i = 0; i < 16; i += 2) {
+        const f2 val = add2(f2(v[i], v[i + 1]), f2(bias_v[mt]));
+        fma2(val, val, f2(sq[16 * hh + i], sq[16 * hh + i + 1])).get(sq[16 * hh + i], sq[16 * hh + i + 1]);
       }
     }
   }
@@ -306,7 +344,8 @@ __device__ __forceinline__ void ep_residual(const ECtx& x, const float* bias, co
       }
       tmem_ld_wait();
 #pragma unroll
-      for (int i = 0; i < 16; ++i) v[i] = (v[i] + bias_v[mt]) * g * rv[i];
+      for (int i = 0; i < 16; i += 2)
+        mul2(mul2(add2(f2(v[i], v[i + 1]), f2(bias_v[mt])), f2(g)), f2(rv[i], rv[i + 1])).get(v[i], v[i + 1]);
       store_row16<FP16>(x.xb, mt * 128 + x.c, c0, v);
     }
     signal_tile();   // x_hat of this tile is in XB
@@ -387,7 +426,11 @@ __device__ __forceinline__ void ep_gate(const ECtx& x, int mt, const float (&xv)
     tmem_ld16(x.gt + mt * 128 + c0, gv);
     tmem_ld_wait();
 #pragma unroll
-    for (int i = 0; i < 16; ++i) mv[i] = fmaf(mv[i] + bm, sigm_pre(fmaf(gv[i], -LOG2E_F, cg)), xv[16 * hh + i]);
+    for (int i = 0; i < 16; i += 2) {
+      f2 e(0.0f), sg(0.0f);
+      sigmoid2(fma2(f2(gv[i], gv[i + 1]), f2(-LOG2E_F), f2(cg)), e, sg);
+      fma2(add2(f2(mv[i], mv[i + 1]), f2(bm)), sg, f2(xv[16 * hh + i], xv[16 * hh + i + 1])).get(mv[i], mv[i + 1]);
+    }
     tmem_st16(x.acc + mt * 128 + c0, mv);   // x' where MLP2 will accumulate
     store_row16<FP16>(x.xb, ch_g, c0, mv);
   }
@@ -416,11 +459,13 @@ __device__ __forceinline__ void scan_gates(const ECtx& x, float (&z)[32], float 
   const uint32_t rm = x.q < 2 ? x.md->m_first[x.half][x.sub] : x.md->m_last[x.half][x.sub];
   const float cz = -bz * LOG2E_F;
 #pragma unroll
-  for (int j = 0; j < 32; ++j) {
-    const float e = ex2_approx(fmaf(z[j], -LOG2E_F, cz));
-    const float sg = rcp_approx(1.0f + e);
-    z[j] = (rm & (1u << j)) ? 0.0f : e * sg;
-    n[j] = sg * (n[j] + bn);
+  for (int j = 0; j < 32; j += 2) {
+    f2 e(0.0f), sg(0.0f);
+    sigmoid2(fma2(f2(z[j], z[j + 1]), f2(-LOG2E_F), f2(cz)), e, sg);
+    mul2(e, sg).get(z[j], z[j + 1]);
+    if (rm & (1u << j)) z[j] = 0.0f;
+    if (rm & (2u << j)) z[j + 1] = 0.0f;
+    mul2(sg, add2(f2(n[j], n[j + 1]), f2(bn))).get(n[j], n[j + 1]);
   }
 }
 // Eq. 2 per channel over this thread's 32 columns (one FMA per hit on the serial
