@@ -18,14 +18,11 @@
 // values lie in its first 128 rows before).  TMEM: two buffers of 256 columns, filled by
 // turns: every product group (the embedding's two, then z and n of 64 channels of both
 // directions) waits only until the epilogue has copied the group before last to registers.
-#include <cuda.h>
-#include <cudaTypedefs.h>
-
 #include <cstring>
 #include <new>
 #include <vector>
 
-#include "tc_epilogue.cuh"
+#include "tiles.cuh"
 
 namespace {
 
@@ -42,7 +39,7 @@ struct CatParams {
   TileSrc src;
   float* pool;          // [B][2 H] endpoint states
   int L, KE, nst;       // layers, 64-row chunks of the Fourier vector, ring stages
-  int last_nk;          // 16-row steps of its last chunk
+  int last_nk;          // 16-row steps of its last chunk: 2 or 4 (E is a multiple of 32)
   uint32_t idesc_mn, idesc_k;   // activations MN-major (shared memory) or K-major (Fourier rows)
   const float *b_e1, *b_e2;     // [128]
   const float* b_in;            // [L][NDC * 256], chunk order
@@ -115,23 +112,22 @@ __global__ void __launch_bounds__(NT, 1) concat_kernel(const __grid_constant__ C
   volatile int* abort = &m->abort_flag;
 
   if (warp == 0) {
-    // TMA producer: the whole warp walks the blocks and waits, one elected lane issues
+    // TMA producer: the whole warp walks the blocks and waits; one lane's copies are let
+    // through by a predicate (see the issuer)
     uint32_t stage = 0, phase = 0;
+    const uint32_t me = elect_one() ? 1u : 0u;
     int issued = 0;
     bool ok = true;
     auto load = [&](int map, int c0, int c1) {
       if (!ok) return;
-      const bool got = mbar_wait(empty0 + 8 * stage, phase ^ 1u, abort, p.wait_ns);
-      if (!__all_sync(0xffffffffu, got)) {
-        if (lane == 0) cat_abort(m, p.err);
+      const uint32_t full = full0 + 8 * stage;
+      if (!mbar_wait(empty0 + 8 * stage, phase ^ 1u, abort, p.wait_ns)) {
+        cat_abort(m, p.err);
         ok = false;
         return;
       }
-      if (elect_one()) {
-        mbar_arrive_expect_tx(full0 + 8 * stage, A_BLOCK);
-        tma_load_2d(ring + stage * A_BLOCK, &p.tm[map], full0 + 8 * stage, c0, c1);
-      }
-      __syncwarp();
+      mbar_arrive_expect_tx_if(full, A_BLOCK, me);
+      tma_load_2d_if(ring + stage * A_BLOCK, &p.tm[map], full, c0, c1, me);
       ++issued;
       if (++stage == (uint32_t)p.nst) {
         stage = 0;
@@ -148,7 +144,8 @@ __global__ void __launch_bounds__(NT, 1) concat_kernel(const __grid_constant__ C
         for (int r = 0; r < 2 * CT_NDC; ++r)   // z, then n, of each chunk
           for (int kc = 0; kc < (l ? 6 : 2); ++kc) load(l ? CM_IN1 : CM_IN0, kc * 64, r * 128);
     }
-    if (!ok) {   // let the copies already issued land before the CTA can exit
+    __syncwarp();
+    if (*abort) {   // let the copies already issued land before the CTA can exit
       volatile int never = 0;
       for (int k = 0; k < p.nst && k < issued; ++k) {
         const int i = issued - 1 - k;
@@ -156,20 +153,22 @@ __global__ void __launch_bounds__(NT, 1) concat_kernel(const __grid_constant__ C
       }
     }
   } else if (warp == 1) {
-    // MMA issuer
+    // MMA issuer: straight-line code for the whole warp, with the instructions of all
+    // lanes but one switched off by a predicate (an elected branch and a vote after each
+    // wait cost twice the time of the products)
     uint32_t stage = 0, phase = 0, g = 0, op_k = 0;
+    const uint32_t me = elect_one() ? 1u : 0u;
     bool ok = true;
     auto wait_bar = [&](uint32_t bar, uint32_t parity) {
-      if (!ok) return;
-      const bool got = mbar_wait(bar, parity, abort, p.wait_ns);
-      if (!__all_sync(0xffffffffu, got)) {
-        if (lane == 0) cat_abort(m, p.err);
+      if (ok && !mbar_wait(bar, parity, abort, p.wait_ns)) {
+        cat_abort(m, p.err);
         ok = false;
       }
-      tc_fence_after();
     };
-    const uint64_t ring_desc = sdesc_sw128(ring, 16, 1024);
-    auto stage_desc = [&]() { return ring_desc + (uint64_t)((stage * A_BLOCK) >> 4); };
+    const uint64_t a_desc = sdesc_sw128(ring, 16, 1024), b_desc = sdesc_sw128(base, B_LBO, B_SBO);
+    const uint32_t a_lo0 = desc_lo(a_desc), a_hi = desc_hi(a_desc), b_lo0 = desc_lo(b_desc), b_hi = desc_hi(b_desc);
+    constexpr uint32_t BSTEP = (2 * B_SBO) >> 4;
+    auto stage_lo = [&]() { return a_lo0 + stage * (A_BLOCK >> 4); };
     auto next_stage = [&]() {
       if (++stage == (uint32_t)p.nst) {
         stage = 0;
@@ -182,24 +181,24 @@ __global__ void __launch_bounds__(NT, 1) concat_kernel(const __grid_constant__ C
       return tmem + (g & 1u) * 256u;
     };
     auto end = [&]() {
-      if (ok && elect_one()) umma_commit(acc_full + 8 * (g & 1u));
-      __syncwarp();
+      umma_commit_if(acc_full + 8 * (g & 1u), ok ? me : 0u);
       ++g;
     };
     auto operand = [&]() { wait_bar(op_bar, op_k++ & 1u); };   // the epilogue's next operand hand-over
-    // kb weight blocks against the activations at byte offset off of shared memory
+    // kb (even) weight blocks against the activations at byte offset off of shared memory
     auto product = [&](uint32_t d, uint32_t off, int kb) {
-      const uint64_t b0 = sdesc_sw128(base + off, B_LBO, B_SBO);
-      constexpr uint32_t BSTEP = (2 * B_SBO) >> 4;
-      for (int kc = 0; kc < kb; ++kc) {
+      uint32_t b_lo = b_lo0 + (off >> 4);
+      for (int kc = 0; kc < kb; kc += 2, b_lo += 8 * BSTEP) {
         wait_bar(full0 + 8 * stage, phase);
-        if (ok && elect_one()) {
-          const uint64_t ad = stage_desc(), bd = b0 + (uint64_t)(kc * 4 * BSTEP);
-#pragma unroll
-          for (int k = 0; k < 4; ++k) umma_f16(d, ad + 2 * k, bd + k * BSTEP, p.idesc_mn, (kc | k) ? 1u : 0u);
-          umma_commit(empty0 + 8 * stage);
-        }
-        __syncwarp();
+        const uint32_t a0 = stage_lo(), e0 = empty0 + 8 * stage;
+        next_stage();
+        wait_bar(full0 + 8 * stage, phase);
+        if (!ok) return;
+        tc_fence_after();
+        umma4_f16_if<BSTEP>(d, a0, a_hi, b_lo, b_hi, p.idesc_mn, kc, me);
+        umma_commit_if(e0, me);
+        umma4_f16_if<BSTEP>(d, stage_lo(), a_hi, b_lo + 4 * BSTEP, b_hi, p.idesc_mn, 1u, me);
+        umma_commit_if(empty0 + 8 * stage, me);
         next_stage();
       }
     };
@@ -208,20 +207,17 @@ __global__ void __launch_bounds__(NT, 1) concat_kernel(const __grid_constant__ C
         const uint32_t d = begin();
         for (int kc = 0; kc < p.KE; ++kc) {
           wait_bar(full0 + 8 * stage, phase);
-          const uint64_t ad = stage_desc();
-          const uint32_t e0 = empty0 + 8 * stage;
+          const uint32_t a0 = stage_lo(), e0 = empty0 + 8 * stage;
           next_stage();
           wait_bar(full0 + 8 * stage, phase);
-          if (ok && elect_one()) {
-            const uint64_t bd = stage_desc();
-            const int nk = kc + 1 < p.KE ? 4 : p.last_nk;
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-              if (k < nk) umma_f16(d, ad + 2 * k, bd + 2 * k, p.idesc_k, (kc | k) ? 1u : 0u);
-            umma_commit(e0);
-            umma_commit(empty0 + 8 * stage);
-          }
-          __syncwarp();
+          if (!ok) break;
+          tc_fence_after();
+          if (kc + 1 < p.KE || p.last_nk == 4)
+            umma4_f16_if<2>(d, a0, a_hi, stage_lo(), a_hi, p.idesc_k, kc, me);
+          else
+            umma2_f16_if<2>(d, a0, a_hi, stage_lo(), a_hi, p.idesc_k, kc, me);
+          umma_commit_if(e0, me);
+          umma_commit_if(empty0 + 8 * stage, me);
           next_stage();
         }
         end();
@@ -241,11 +237,12 @@ __global__ void __launch_bounds__(NT, 1) concat_kernel(const __grid_constant__ C
           end();
         }
     }
-    // no MMA may still run when TMEM is released
-    if (elect_one()) umma_commit(drain_bar);
     __syncwarp();
+    // no MMA may still run when TMEM is released (by the lane that issued them)
+    umma_commit_if(drain_bar, me);
     volatile int never = 0;
     mbar_wait(drain_bar, 0, &never, CT_DRAIN_NS);
+    __syncwarp();
   } else if (warp < 2 + NE / 32) {
     // Epilogue.  The warps run decoupled: each arrives on the hand-over barriers itself
     // (16 arrivals).  One operand barrier is enough: between two operand hand-overs every
@@ -348,102 +345,6 @@ __global__ void __launch_bounds__(NT, 1) concat_kernel(const __grid_constant__ C
   }
 }
 
-// ------------------------------------------------------------------ Fourier rows
-// Sec. 3.2, for the hits of a slab: row 64 s + column holds the hit's Fourier vector
-// (per feature 16 sines, 16 cosines); columns without a hit hold zeros.  One thread per
-// (column, feature), the argument as in rows.cu (an unevaluated sum of two floats,
-// reduced modulo 2 exactly; with scales 2^(k/3) nine of 16 evaluated, the others by
-// one double-angle step).
-template <bool FP16>
-__global__ void __launch_bounds__(256) fourier_slab_kernel(const TileSrc src, const __grid_constant__ tf_shape s,
-                                                           uint16_t* __restrict__ e) {
-  __shared__ int64_t row_s[SLAB];
-  const int n_slabs = *src.n_slabs;
-  for (int sl = blockIdx.x; sl < n_slabs; sl += gridDim.x) {
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      const int lane = threadIdx.x;
-      const int2 d = src.slab[sl];
-      int n = 0;
-      int64_t r = 0;
-      if (lane < d.y) {
-        const int b = src.order[d.x + lane];
-        n = src.n_hits[b];
-        if (n < 1 || n > s.T) n = 0;
-        r = src.offs ? src.offs[b] : (int64_t)b * s.T;
-      }
-      int end = n;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int u = __shfl_up_sync(0xffffffffu, end, o);
-        if (lane >= o) end += u;
-      }
-      for (int t = 0; t < n; ++t) row_s[end - n + t] = r + t;
-      const int all = __shfl_sync(0xffffffffu, end, 31);
-      for (int c = all + lane; c < SLAB; c += 32) row_s[c] = -1;
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < SLAB * s.F; i += 256) {
-      const int c = i / s.F, f = i - c * s.F;
-      uint4* o = reinterpret_cast<uint4*>(e + ((size_t)sl * SLAB + c) * s.E + f * 2 * TRACKFIT_MAX_FOURIER);
-      const int64_t row = row_s[c];
-      if (row < 0) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) o[q] = make_uint4(0u, 0u, 0u, 0u);
-        continue;
-      }
-      const float v = src.hits[row * s.F + f];
-      const float mn = -s.feat_min[f], ih = s.feat_inv_range[f];
-      const float dh = v + mn, bv = dh - v, dl = (v - (dh - bv)) + (mn - bv);
-      const float uh = dh * ih;
-      const float ul = fmaf(dh, ih, -uh) + fmaf(dh, s.feat_inv_lo[f], dl * ih);
-      float sv[TRACKFIT_MAX_FOURIER], cv[TRACKFIT_MAX_FOURIER];
-#pragma unroll
-      for (int k = 0; k < TRACKFIT_MAX_FOURIER; ++k) {
-        if (src.scale_doubling && (k % 6) >= 3) {   // s_k = 2 s_{k-3}
-          sv[k] = 2.0f * sv[k - 3] * cv[k - 3];
-          cv[k] = (cv[k - 3] - sv[k - 3]) * (cv[k - 3] + sv[k - 3]);
-          continue;
-        }
-        const float sk = s.scale[k], xh = uh * sk, xl = fmaf(uh, sk, -xh) + ul * sk;
-        sincospif((xh - 2.0f * rintf(0.5f * xh)) + xl, &sv[k], &cv[k]);
-      }
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        o[q] = make_uint4(pack2<FP16>(sv[8 * q], sv[8 * q + 1]), pack2<FP16>(sv[8 * q + 2], sv[8 * q + 3]),
-                          pack2<FP16>(sv[8 * q + 4], sv[8 * q + 5]), pack2<FP16>(sv[8 * q + 6], sv[8 * q + 7]));
-        o[2 + q] = make_uint4(pack2<FP16>(cv[8 * q], cv[8 * q + 1]), pack2<FP16>(cv[8 * q + 2], cv[8 * q + 3]),
-                              pack2<FP16>(cv[8 * q + 4], cv[8 * q + 5]), pack2<FP16>(cv[8 * q + 6], cv[8 * q + 7]));
-      }
-    }
-  }
-}
-
-// 16-bit matrix [rows][cols] row-major -> tensor map of 64-column x 128-row boxes with
-// 128-byte swizzle (out-of-range elements read as zero).
-bool cat_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, bool fp16) {
-  void* f = nullptr;
-  cudaDriverEntryPointQueryResult q;
-  if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-      q != cudaDriverEntryPointSuccess)
-    return false;
-  cuuint64_t dims[2] = {cols, rows}, strides[1] = {cols * 2};
-  cuuint32_t box[2] = {64, 128}, es[2] = {1, 1};
-  return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(f)(
-             m, fp16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr),
-             dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-uint16_t cat_16(float f, bool fp16) {
-  if (fp16) {
-    const __half v = __float2half_rn(f);
-    return *reinterpret_cast<const uint16_t*>(&v);
-  }
-  const __nv_bfloat16 v = __float2bfloat16_rn(f);
-  return *reinterpret_cast<const uint16_t*>(&v);
-}
-
 }  // namespace
 
 struct tf_cat_state {
@@ -503,8 +404,8 @@ int tf_cat_create(trackfit_ctx* h, const float* W, tf_cat_state** out) {
   std::vector<uint16_t> w(D * E + D * D + rows * D + rows * 2 * H);
   std::vector<float> b(2 * D + 2 * rows, 0.0f);
   size_t at = 0;
-  for (size_t i = 0; i < D * E; ++i) w[at++] = cat_16(W[o.emb_w1 + i], fp16);
-  for (size_t i = 0; i < D * D; ++i) w[at++] = cat_16(W[o.emb_w2 + i], fp16);
+  for (size_t i = 0; i < D * E; ++i) w[at++] = to_16(W[o.emb_w1 + i], fp16);
+  for (size_t i = 0; i < D * D; ++i) w[at++] = to_16(W[o.emb_w2 + i], fp16);
   for (size_t i = 0; i < D; ++i) {
     b[i] = W[o.emb_b1 + i];
     b[D + i] = W[o.emb_b2 + i];
@@ -517,7 +418,7 @@ int tf_cat_create(trackfit_ctx* h, const float* W, tf_cat_state** out) {
       const size_t src = (2 * dir + n) * H + ch;
       for (size_t k = 0; k < I; ++k) {
         const size_t kk = l ? ((k / 64) & 1) * H + (k / 128) * 64 + (k & 63) : k;
-        w[at++] = cat_16(W[lo.w_in + src * I + kk], fp16);
+        w[at++] = to_16(W[lo.w_in + src * I + kk], fp16);
       }
       b[2 * D + l * rows + r] = W[lo.b_in + src];
     }
@@ -533,14 +434,10 @@ int tf_cat_create(trackfit_ctx* h, const float* W, tf_cat_state** out) {
   p.b_e1 = db;
   p.b_e2 = db + D;
   p.b_in = db + 2 * D;
-  // tracks of a chunk: a slab holds at least 64 / T full-length tracks (or 16 tracks),
-  // and each of a segment's 256 tracks' last slab may be part-filled
-  const int64_t per = SLAB / s.T < TF_SLAB_TRACKS ? SLAB / s.T : TF_SLAB_TRACKS;
-  auto slabs = [&](int64_t n) { return (n + per - 1) / per + n / 256 + 2; };
   int64_t chunk = 1 << 20;
-  while (chunk > 1024 && (size_t)slabs(chunk) * SLAB * E * 2 + (size_t)chunk * 2 * H * 4 > CT_WS_BUDGET) chunk -= 1024;
+  while (chunk > 1024 && (size_t)slab_bound(chunk, s.T) * SLAB * E * 2 + (size_t)chunk * 2 * H * 4 > CT_WS_BUDGET) chunk -= 1024;
   c->chunk = chunk;
-  const int64_t cap = (slabs(chunk) + 1) / 2 * TILE;
+  const int64_t cap = (slab_bound(chunk, s.T) + 1) / 2 * TILE;
   if (st == TRACKFIT_OK) st = tf_status_from_cuda(tf_malloc(&c->pack, tf_pack_bytes(chunk)));
   if (st == TRACKFIT_OK) st = tf_status_from_cuda(tf_malloc((void**)&c->four, (size_t)cap * E * 2));
   if (st == TRACKFIT_OK) st = tf_status_from_cuda(tf_malloc((void**)&c->pool, (size_t)chunk * 2 * H * 4));
@@ -549,9 +446,9 @@ int tf_cat_create(trackfit_ctx* h, const float* W, tf_cat_state** out) {
   if (st == TRACKFIT_OK) st = tf_status_from_cuda(cudaMemset(c->four, 0, (size_t)cap * E * 2));
   if (st != TRACKFIT_OK) return st;
   const uint16_t *we2 = dw + D * E, *w0 = we2 + D * D, *w1 = w0 + rows * D;
-  if (!cat_map(&p.tm[CM_F], c->four, (uint64_t)cap, E, fp16) || !cat_map(&p.tm[CM_E1], dw, D, E, fp16) ||
-      !cat_map(&p.tm[CM_E2], we2, D, D, fp16) || !cat_map(&p.tm[CM_IN0], w0, rows, D, fp16) ||
-      !cat_map(&p.tm[CM_IN1], w1, rows, 2 * H, fp16))
+  if (!tile_map(&p.tm[CM_F], c->four, (uint64_t)cap, E, fp16) || !tile_map(&p.tm[CM_E1], dw, D, E, fp16) ||
+      !tile_map(&p.tm[CM_E2], we2, D, D, fp16) || !tile_map(&p.tm[CM_IN0], w0, rows, D, fp16) ||
+      !tile_map(&p.tm[CM_IN1], w1, rows, 2 * H, fp16))
     return TRACKFIT_ERR_CUDA;
   for (auto k : {concat_kernel<false>, concat_kernel<true>})
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->smem) != cudaSuccess)
@@ -568,9 +465,6 @@ int tf_cat_forward(trackfit_ctx* h, tf_cat_state* c, uint64_t wait_ns, const flo
   p.err = h->d_err;
   p.wait_ns = wait_ns;
   p.src.T = s.T;
-  p.src.scale_doubling = 1;
-  for (int k = 0; k + 3 < TRACKFIT_MAX_FOURIER; ++k)
-    if (s.scale[k + 3] != 2.0f * s.scale[k]) p.src.scale_doubling = 0;
   const tf_pack pk = tf_pack_in(c->pack, c->chunk);
   p.src.slab = pk.slab;
   p.src.order = pk.order;
@@ -582,12 +476,8 @@ int tf_cat_forward(trackfit_ctx* h, tf_cat_state* c, uint64_t wait_ns, const flo
     p.src.n_hits = n_hits + c0;
     p.pool = out_pool ? out_pool + c0 * s.P : c->pool;
     cudaError_t e = tf_plan(p.src.n_hits, nb, s.T, c->nsm, pk.order, pk.slab, pk.n_slabs, st);
-    const unsigned fgrid = (unsigned)(nb < 8 * c->nsm ? nb : 8 * c->nsm);
+    if (e == cudaSuccess) e = fourier_slabs(p.src, s, nb, c->nsm, c->four, st);
     if (e == cudaSuccess) {
-      if (fp16)
-        fourier_slab_kernel<true><<<fgrid, 256, 0, st>>>(p.src, s, c->four);
-      else
-        fourier_slab_kernel<false><<<fgrid, 256, 0, st>>>(p.src, s, c->four);
       tf_prof_begin(h, st);
       if (fp16)
         concat_kernel<true><<<c->nsm, NT, c->smem, st>>>(p);

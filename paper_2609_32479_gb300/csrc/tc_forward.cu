@@ -38,9 +38,8 @@
 namespace {
 
 constexpr int A_STAGE = 2 * A_BLOCK;      // a pipeline stage holds two consecutive blocks
-constexpr int MAX_SCHED = 2048;           // schedule entries per tile
+constexpr int MAX_SCHED = 1024;           // schedule steps per tile
 constexpr int MISC_BYTES = 10240;
-constexpr int SCHED_BYTES = 2 * MAX_SCHED * 4;   // both schedule tables, copied to shared memory
 constexpr int MAX_STAGES = 8;
 constexpr int64_t MAXB = TF_PACK_TRACKS;  // tracks per launch chunk
 constexpr int64_t POOL_TRACKS = 1048576;  // tracks per launch chunk when the pooled means go to the internal buffer
@@ -55,19 +54,25 @@ enum { BSEL_XB = 0, BSEL_HB = 1 };
 // used alternately) or hb_bar (C_HB).
 enum { W_NONE = 0, W_E = 1, W_H = 2 };
 enum { C_NONE = 0, C_ACC = 1, C_HB = 2 };
-// bits of an MMA schedule entry
-constexpr uint32_t S_NK4 = 1u << 16, S_ACC = 1u << 17, S_C_ACC = 1u << 18, S_C_HB = 1u << 19, S_W_E = 1u << 20,
-                   S_W_H = 1u << 21;
+// A schedule step: two consecutive 64-k blocks of one product (a weight row block and
+// K columns col, col + 64), one ring stage at d_model 256.  TAIL: the last 32 k-rows of the
+// Fourier operand, a half block each of the step's one (d_model 128) or two 128-channel
+// tiles.  prod: map | col/64 << 4 | row << 8; mma: the B operand's offset / 16 in the
+// activation buffers | flags << 16, with the accumulator columns / 128 in flags' low bits.
+struct Step {
+  uint32_t prod, mma;
+};
+constexpr uint32_t S_COL = 3u << 16, S_ACC = 1u << 18, S_TAIL = 1u << 19, S_W_E = 1u << 20, S_W_H = 1u << 21,
+                   S_W_X = 1u << 22, S_C_ACC = 1u << 23, S_C_HB = 1u << 24, S_TILE = 1u << 25;
+
+constexpr int SCHED_BYTES = MAX_SCHED * (int)sizeof(Step);   // the schedule, copied to shared memory
 
 struct TcParams {
   CUtensorMap tm[NMAPS];
   TileSrc src;
   float* pool;   // [B][D] pooled means (the caller's buffer or an internal one)
   float* xs;
-  // per block: sched_p map | col/64 << 4 | row << 8, sched_m b offset | bsel << 13 |
-  // tcol/128 << 14 | S_* flags; two tables for d_model 128 (one tile, two tiles)
-  const uint32_t* sched_p;
-  const uint32_t* sched_m;
+  const Step* sched;   // the steps of a tile (d_model 128: then those of two tiles)
   int n_sched, n_sched2;
   const float* b_e1;
   const float* b_e2;
@@ -102,7 +107,8 @@ struct Misc {
 static_assert(sizeof(Misc) <= MISC_BYTES, "misc region too small");
 
 // The static sequence of 128x64 weight blocks of one tile, in the order the MMA
-// issuer consumes them.  f(map, row, col, nk, tmem_col, bsel, bk, acc, wait, commit):
+// issuer consumes them, two blocks a step (waits fall on the first of a step, commits on
+// the second).  f(map, row, col, nk, tmem_col, bsel, bk, acc, wait, commit):
 // nk MMAs of K=16 read the block, accumulate into TMEM columns tmem_col, with
 // the activation operand bsel starting at k-row bk; acc = accumulate onto the
 // existing accumulator; wait / commit = hand-overs (W_*, C_*).
@@ -112,13 +118,15 @@ static_assert(sizeof(Misc) <= MISC_BYTES, "misc region too small");
 // issuer computes z/n of chunk k+1 into the same TMEM columns, and the merge
 // product of chunk k follows once its states h(k) are in shared memory.
 template <class F>
-__host__ __device__ inline void walk_tile(const TcParams& p, F&& f) {   // d_model 256
+inline void walk_tile(const TcParams& p, F&& f) {   // d_model 256
   // the embedding's first product goes to the z/n columns, so it can run while
   // the epilogue still pools the previous tile from columns 0..
   for (int mt = 0; mt < 2; ++mt)
-    for (int kc = 0; kc < 3; ++kc)
-      f(MAP_E1, mt * 128, kc * 64, kc == 2 ? 2 : 4, 256 + mt * 128, BSEL_HB, kc * 64, kc > 0,
-        (mt == 0 && kc == 0) ? W_E : W_NONE, (mt == 1 && kc == 2) ? C_ACC : C_NONE);
+    for (int kc = 0; kc < 2; ++kc)
+      f(MAP_E1, mt * 128, kc * 64, 4, 256 + mt * 128, BSEL_HB, kc * 64, kc > 0, (mt == 0 && kc == 0) ? W_E : W_NONE,
+        C_NONE);
+  for (int mt = 0; mt < 2; ++mt)   // its last 32 k-rows
+    f(MAP_E1, mt * 128, 128, 2, 256 + mt * 128, BSEL_HB, 128, true, W_NONE, mt == 1 ? C_ACC : C_NONE);
   for (int mt = 0; mt < 2; ++mt)   // committed per 128-channel tile, like MLP2
     for (int kc = 0; kc < 4; ++kc)
       f(MAP_E2, mt * 128, kc * 64, 4, mt * 128, BSEL_XB, kc * 64, kc > 0, (mt == 0 && kc == 0) ? W_E : W_NONE,
@@ -231,11 +239,8 @@ __global__ void __launch_bounds__(NT, 1) tc_forward_kernel(const __grid_constant
     m->abort_flag = 0;
     fence_mbar_init();
   }
-  uint32_t* sched_s = reinterpret_cast<uint32_t*>(gbase + p.off_misc + MISC_BYTES);   // [2][MAX_SCHED]
-  for (int i = threadIdx.x; i < p.n_sched; i += blockDim.x) {
-    sched_s[i] = p.sched_p[i];
-    sched_s[MAX_SCHED + i] = p.sched_m[i];
-  }
+  Step* sched_s = reinterpret_cast<Step*>(gbase + p.off_misc + MISC_BYTES);
+  for (int i = threadIdx.x; i < p.n_sched; i += blockDim.x) sched_s[i] = p.sched[i];
   if (warp == 1) {
     tmem_alloc(smem_u32(&m->tmem_base), 512);
     tmem_relinquish();
@@ -252,157 +257,110 @@ __global__ void __launch_bounds__(NT, 1) tc_forward_kernel(const __grid_constant
   volatile int* abort = &m->abort_flag;
 
   if (warp == 0) {
-    // TMA producer: two consecutive 16 KB weight blocks per stage, in schedule
-    // order (the CTA's block sequence runs on across tiles; a final odd block
-    // occupies a stage alone).  The whole warp walks the schedule and waits; one
-    // elected lane issues (a loop run by a lone lane issues far slower).
+    // TMA producer: a step's two 16 KB weight blocks per stage, in schedule order.  The
+    // whole warp walks the schedule and waits; one lane's copies are let through by a
+    // predicate (see the issuer).
     uint32_t stage = 0, phase = 0;
+    const uint32_t me = elect_one() ? 1u : 0u;
     bool ok = true;
-    int issued = 0, half = 0;
-    int my_tiles = 0;
-    for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) ++my_tiles;
-    const int total = my_tiles * p.n_sched;
+    int issued = 0;
     for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
       for (int i = 0; i < p.n_sched; ++i) {
-        const uint32_t e = sched_s[i];
-        if (half == 0) {
-          const bool got = mbar_wait(empty0 + 8 * stage, phase ^ 1u, abort, p.wait_ns);
-          if (!__all_sync(0xffffffffu, got)) {
-            if (lane == 0) set_abort(&m->abort_flag, p.err);
-            ok = false;
-            break;
-          }
+        const Step e = sched_s[i];
+        const CUtensorMap* map = &p.tm[e.prod & 15u];
+        const int c0 = (int)((e.prod >> 4) & 15u) * 64, c1 = (int)(e.prod >> 8);
+        const bool tail = e.mma & S_TAIL;
+        const uint32_t full = full0 + 8 * stage, dst = ab + stage * A_STAGE;
+        if (!mbar_wait(empty0 + 8 * stage, phase ^ 1u, abort, p.wait_ns)) {
+          set_abort(&m->abort_flag, p.err);
+          ok = false;
+          break;
         }
-        if (elect_one()) {
-          if (half == 0) mbar_arrive_expect_tx(full0 + 8 * stage, issued + 1 < total ? A_STAGE : A_BLOCK);
-          tma_load_2d(ab + stage * A_STAGE + half * A_BLOCK, &p.tm[e & 15u], full0 + 8 * stage,
-                      (int)((e >> 4) & 15u) * 64, (int)(e >> 8));
-        }
-        __syncwarp();
+        mbar_arrive_expect_tx_if(full, A_STAGE, me);
+        tma_load_2d_if(dst, map, full, c0, c1, me);
+        tma_load_2d_if(dst + A_BLOCK, map, full, tail ? c0 : c0 + 64, tail ? c1 + 128 : c1, me);
         ++issued;
-        if (++half == 2) {
-          half = 0;
-          if (++stage == (uint32_t)p.nst) {
-            stage = 0;
-            phase ^= 1u;
-          }
+        if (++stage == (uint32_t)p.nst) {
+          stage = 0;
+          phase ^= 1u;
         }
       }
     }
-    if (!ok) {
+    __syncwarp();
+    if (*abort) {
       // let the copies already issued land before the CTA can exit
       volatile int never = 0;
-      const int used = (issued + 1) / 2;
-      for (int k = 0; k < p.nst && k < used; ++k) {
-        const int i = used - 1 - k;
+      for (int k = 0; k < p.nst && k < issued; ++k) {
+        const int i = issued - 1 - k;
         mbar_wait(full0 + 8 * (i % p.nst), (uint32_t)((i / p.nst) & 1), &never, DRAIN_NS);
       }
     }
   } else if (warp == 1) {
-    // MMA issuer, run by the whole warp with one elected lane issuing.  One
-    // iteration per stage (two consecutive schedule blocks, 8 MMAs): the stage's
-    // barrier is tested without blocking first, and both blocks go out in one
-    // elected run unless an epilogue hand-over falls between them, so the
-    // per-iteration bookkeeping stays short next to the tensor pipe's queue.
-    uint32_t stage = 0, phase = 0, eh_phase = 0, e_k = 0, e_phase0 = 0, e_phase1 = 0;
+    // MMA issuer.  It must hand the tensor pipe 8 products every 512 cycles while five
+    // warps share its scheduler, so its own instructions count: with a branch around an
+    // elected lane, a vote after each wait and a block a time it took 755 cycles for 4
+    // products beside busy warps (N = 64 products took as long as N = 128).  So the whole
+    // warp runs one straight line a step, the instructions of all lanes but one are
+    // switched off by a predicate, and the next step's entry is loaded ahead: 314
+    // cycles for 4.
+    uint32_t stage = 0, phase = 0, e_k = 0, h_k = 0, a_k = 0;
+    const uint32_t me = elect_one() ? 1u : 0u;
     bool ok = true;
-    int my_tiles = 0;
-    for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) ++my_tiles;
-    const int total = my_tiles * p.n_sched;
-    const int n_stages = (total + 1) >> 1;
-    const uint64_t a_desc0 = sdesc_sw128(ab, 16, 1024);
-    const uint64_t b_desc_xb = sdesc_sw128(xb, B_LBO, B_SBO), b_desc_hb = sdesc_sw128(hb, B_LBO, B_SBO);
+    const uint64_t a_desc = sdesc_sw128(ab, 16, 1024), b_desc = sdesc_sw128(base, B_LBO, B_SBO);
+    const uint32_t a_lo0 = desc_lo(a_desc), a_hi = desc_hi(a_desc), b_lo0 = desc_lo(b_desc), b_hi = desc_hi(b_desc);
     constexpr uint32_t BSTEP = (2 * B_SBO) >> 4;
-    const uint32_t* sm_tab = sched_s + MAX_SCHED;
     const uint32_t idesc = p.idesc;
-    auto wait_bar = [&](uint32_t bar, uint32_t& ph, bool spin) -> bool {
-      const bool got = spin ? mbar_wait_spin(bar, ph, abort, p.wait_ns) : mbar_wait(bar, ph, abort, p.wait_ns);
-      if (!__all_sync(0xffffffffu, got)) {
-        if (lane == 0) set_abort(&m->abort_flag, p.err);
-        return false;
+    auto wait_bar = [&](uint32_t bar, uint32_t parity) {
+      if (!mbar_wait(bar, parity, abort, p.wait_ns)) {
+        set_abort(&m->abort_flag, p.err);
+        ok = false;
       }
-      ph ^= 1u;
-      return true;
     };
-    auto handover = [&](uint32_t e) -> bool {
-      if (e & S_W_E) {   // the k-th W_E hand-over arrives on e_bar[k % 2]
-        const bool got = (e_k & 1u) ? wait_bar(e_bar1, e_phase1, false) : wait_bar(e_bar0, e_phase0, false);
-        if (!got) return false;
-        ++e_k;
-      } else if (!wait_bar(eh_bar, eh_phase, false)) {
-        return false;
-      }
-      tc_fence_after();
-      return true;
-    };
-    // The k-th accumulator commit goes to acc_bar[k % 2] (some commits come in
-    // pairs with no epilogue hand-over between them; see the epilogue).  The
-    // count is kept by the whole warp: the barrier of a block's commit, and the
-    // count advanced past it.
-    uint32_t acc_k = 0;
-    auto acc_for = [&](uint32_t e) -> uint32_t {
-      const uint32_t b = (acc_k & 1u) ? acc_bar1 : acc_bar0;
-      if (e & S_C_ACC) ++acc_k;
-      return b;
-    };
-    // the MMAs and group commits of one block (elected lane only)
-    auto issue = [&](uint32_t e, uint64_t ad, uint32_t acc_b) {
-      const uint64_t bd = ((e >> 13) & 1u ? b_desc_hb : b_desc_xb) + (uint64_t)(e & 0x1FFFu);
-      const uint32_t d = tmem + ((e >> 14) & 3u) * 128u;
-      const uint32_t nk4 = e & S_NK4;
-      umma_f16(d, ad, bd, idesc, e & S_ACC);
-      umma_f16(d, ad + 2, bd + BSTEP, idesc, 1u);
-      umma_f16_if(d, ad + 4, bd + 2 * BSTEP, idesc, 1u, nk4);
-      umma_f16_if(d, ad + 6, bd + 3 * BSTEP, idesc, 1u, nk4);
-      umma_commit_if(acc_b, e & S_C_ACC);
-      umma_commit_if(hb_bar, e & S_C_HB);
-    };
-    int i0 = 0;   // schedule index of the stage's first block
-    for (int sg = 0; sg < n_stages; ++sg) {
-      int i1 = i0 + 1;
-      if (i1 == p.n_sched) i1 = 0;
-      const bool two = 2 * sg + 1 < total;
-      const uint32_t e0 = sm_tab[i0], e1 = two ? sm_tab[i1] : 0u;
-      i0 = i1 + 1;
-      if (i0 >= p.n_sched) i0 -= p.n_sched;
-      const uint32_t ab0 = acc_for(e0), ab1 = acc_for(e1);   // (e1 = 0 commits nothing)
-      if ((e0 & (S_W_E | S_W_H)) && !(ok = handover(e0))) break;
-      if (!mbar_test_wait(full0 + 8 * stage, phase)) {
-        uint32_t ph = phase;
-        if (!(ok = wait_bar(full0 + 8 * stage, ph, false))) break;
-      }
-      tc_fence_after();
-      const uint64_t ad0 = a_desc0 + (uint64_t)((stage * A_STAGE) >> 4);
-      const uint64_t ad1 = ad0 + (uint64_t)(A_BLOCK >> 4);
-      const uint32_t empty = empty0 + 8 * stage;
-      if (e1 & (S_W_E | S_W_H)) {   // a hand-over between the two blocks
-        if (elect_one()) issue(e0, ad0, ab0);
-        __syncwarp();
-        if (!(ok = handover(e1))) break;
-        if (elect_one()) {
-          issue(e1, ad1, ab1);
-          umma_commit(empty);
+    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+      uint32_t e = sched_s[0].mma;
+      for (int i = 0; i < p.n_sched; ++i) {
+        const uint32_t en = sched_s[i + 1 < p.n_sched ? i + 1 : 0].mma;
+        if (e & S_W_E) {   // the k-th W_E hand-over arrives on e_bar[k % 2]
+          wait_bar(e_bar0 + 8 * (e_k & 1u), (e_k >> 1) & 1u);
+          ++e_k;
+        } else if (e & S_W_H) {
+          wait_bar(eh_bar, h_k & 1u);
+          ++h_k;
         }
-        __syncwarp();
-      } else {
-        if (elect_one()) {
-          issue(e0, ad0, ab0);
-          if (two) issue(e1, ad1, ab1);
-          umma_commit(empty);
+        wait_bar(full0 + 8 * stage, phase);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t a_lo = a_lo0 + stage * (A_STAGE >> 4), b_lo = b_lo0 + (e & 0xFFFFu);
+        const uint32_t d = tmem + ((e & S_COL) >> 16) * 128u;
+        if (!(e & S_TAIL)) {
+          umma4_f16_if<BSTEP>(d, a_lo, a_hi, b_lo, b_hi, idesc, e & S_ACC, me);
+          umma4_f16_if<BSTEP>(d, a_lo + (A_BLOCK >> 4), a_hi, b_lo + 4 * BSTEP, b_hi, idesc, 1u, me);
+        } else {
+          umma2_f16_if<BSTEP>(d, a_lo, a_hi, b_lo, b_hi, idesc, 1u, me);
+          umma2_f16_if<BSTEP>(d + 128u, a_lo + (A_BLOCK >> 4), a_hi, b_lo, b_hi, idesc, 1u, me);
         }
-        __syncwarp();
-      }
-      if (++stage == (uint32_t)p.nst) {
-        stage = 0;
-        phase ^= 1u;
+        umma_commit_if(empty0 + 8 * stage, me);
+        // The k-th accumulator commit goes to acc_bar[k % 2] (some commits come in
+        // pairs with no epilogue hand-over between them; see the epilogue).
+        if (e & S_C_ACC) {
+          umma_commit_if(acc_bar0 + 8 * (a_k & 1u), me);
+          ++a_k;
+        } else if (e & S_C_HB) {
+          umma_commit_if(hb_bar, me);
+        }
+        e = en;
+        if (++stage == (uint32_t)p.nst) {
+          stage = 0;
+          phase ^= 1u;
+        }
       }
     }
-    // no MMA may still run when TMEM is released (the elected lane is the one
-    // that issued them)
-    if (elect_one()) umma_commit(drain_bar);
     __syncwarp();
+    // no MMA may still run when TMEM is released (by the lane that issued them)
+    umma_commit_if(drain_bar, me);
     volatile int never = 0;
     mbar_wait(drain_bar, 0, &never, DRAIN_NS);
+    __syncwarp();
   } else if (warp < 2 + NE / 32) {
     ECtx x;
     x.xb = xb;
@@ -592,30 +550,6 @@ __global__ void __launch_bounds__(NT, 1) tc_forward_kernel(const __grid_constant
 
 #include "tc_pair.cuh"
 
-// ------------------------------------------------------------------ schedule
-// One thread expands walk_tile, or walk_pair for nt tiles, into the compact per-block
-// entries read by the producer and the MMA issuer (identical for every tile).
-__global__ void build_schedule(const __grid_constant__ TcParams p, int nt, uint32_t* sp, uint32_t* sm, int* count) {
-  int n = 0;
-  auto put = [&](int u, int map, int row, int col, int nk, int tcol, int bsel, int bk, int acc, int wait, int commit) {
-    if (n < MAX_SCHED) {
-      sp[n] = (uint32_t)map | ((uint32_t)(col >> 6) << 4) | ((uint32_t)row << 8);
-      sm[n] = (uint32_t)(((bk >> 3) * B_SBO) >> 4) | ((uint32_t)bsel << 13) | ((uint32_t)(tcol >> 7) << 14) |
-              (nk == 4 ? S_NK4 : 0u) | (acc ? S_ACC : 0u) | (commit == C_ACC ? S_C_ACC : 0u) |
-              (commit == C_HB ? S_C_HB : 0u) | ((wait & W_E) ? S_W_E : 0u) | ((wait & W_H) ? S_W_H : 0u) |
-              ((wait & W_X) ? S_W_X : 0u) | (u ? S_TILE : 0u);
-    }
-    ++n;
-  };
-  if (p.D == 128)
-    walk_pair(p.L, p.NDC, p.ROWS_IN, nt, put);
-  else
-    walk_tile(p, [&](int map, int row, int col, int nk, int tcol, int bsel, int bk, int acc, int wait, int commit) {
-      put(0, map, row, col, nk, tcol, bsel, bk, acc, wait, commit);
-    });
-  *count = n;
-}
-
 // ------------------------------------------------------------------ UMMA probe
 // D[128][128] = A[128][K] * B[K][128] through the same TMA / descriptor / TMEM
 // path as the fused kernel (test hook for the operand layouts).
@@ -751,7 +685,7 @@ struct tf_tc_state {
   float *b_e1 = nullptr, *b_e2 = nullptr, *g = nullptr, *b_in = nullptr, *b_m = nullptr, *b_1 = nullptr,
         *b_2 = nullptr;
   void* pack = nullptr;   // packing buffers for MAXB tracks
-  uint32_t* sched = nullptr;   // [4][MAX_SCHED]: producer and MMA entries of one tile, then of two (d_model 128)
+  Step* sched = nullptr;   // steps of one tile, then (d_model 128) of two
   int n_sched = 0, n_sched2 = 0;
   float* xs = nullptr;
   uint8_t* fbuf = nullptr;
@@ -761,11 +695,47 @@ struct tf_tc_state {
   CUtensorMap tm[NMAPS];
 };
 
+// Steps of a tile at d_model 128: the embedding's 2 + 1, a layer's products.
+static int pair_steps(int L, int NDC) { return 3 + L * (3 * NDC + 3); }
+
+// The steps of one tile (nt = 1) or of two in turn (d_model 128, nt = 2): walk_tile's or
+// walk_pair's blocks, two at a time.
+static std::vector<Step> build_schedule(int D, int L, int NDC, int ROWS_IN, int nt) {
+  std::vector<Step> out;
+  bool second = false;
+  auto put = [&](int u, int map, int row, int col, int nk, int tcol, int bsel, int bk, int acc, int wait, int commit) {
+    const uint32_t commits = (commit == C_ACC ? S_C_ACC : 0u) | (commit == C_HB ? S_C_HB : 0u);
+    if (!second) {
+      const int off = D == 128 ? u * P_TILE + (bsel == BSEL_HB ? P_HB : P_XB) : (bsel == BSEL_HB ? D * 256 : 0);
+      out.push_back({(uint32_t)map | ((uint32_t)(col >> 6) << 4) | ((uint32_t)row << 8),
+                     (uint32_t)((off + (bk >> 3) * B_SBO) >> 4) | ((uint32_t)(tcol >> 7) << 16) | (acc ? S_ACC : 0u) |
+                         (nk == 2 ? S_TAIL : 0u) | ((wait & W_E) ? S_W_E : 0u) | ((wait & W_H) ? S_W_H : 0u) |
+                         ((wait & W_X) ? S_W_X : 0u) | (u ? S_TILE : 0u)});
+    }
+    out.back().mma |= commits;
+    second = !second && !(D == 128 && nk == 2);   // d_model 128: the tail is a step of one block
+  };
+  if (D == 128) {
+    walk_pair(L, NDC, ROWS_IN, nt, put);
+  } else {
+    TcParams q;
+    std::memset(&q, 0, sizeof(q));
+    q.D = D;
+    q.L = L;
+    q.NDC = NDC;
+    q.ROWS_IN = ROWS_IN;
+    walk_tile(q, [&](int map, int row, int col, int nk, int tcol, int bsel, int bk, int acc, int wait, int commit) {
+      put(0, map, row, col, nk, tcol, bsel, bk, acc, wait, commit);
+    });
+  }
+  return out;
+}
+
 struct ScheduleCounter {   // a callable for walk_tile on either side
   int64_t c[6] = {0, 0, 0, 0, 0, 0};
   uint8_t* codes = nullptr;   // optional: per block wait | commit << 2, in order
   int64_t cap = 0;
-  __host__ __device__ void operator()(int, int, int, int nk, int, int, int, int, int wait, int commit) {
+  void operator()(int, int, int, int nk, int, int, int, int, int wait, int commit) {
     if (c[0] < cap) codes[c[0]] = (uint8_t)(wait | (commit << 2));
     ++c[0];
     c[1] += nk;
@@ -774,7 +744,7 @@ struct ScheduleCounter {   // a callable for walk_tile on either side
     c[4] += commit == C_ACC;
     c[5] += commit == C_HB;
   }
-  __host__ __device__ void operator()(int, int map, int row, int col, int nk, int tcol, int bsel, int bk, int acc,
+  void operator()(int, int map, int row, int col, int nk, int tcol, int bsel, int bk, int acc,
                                       int wait, int commit) {   // walk_pair
     (*this)(map, row, col, nk, tcol, bsel, bk, acc, wait, commit);
   }
@@ -849,8 +819,7 @@ int tf_tc_create(trackfit_ctx* h, const float* W) {
   int smem_optin = 0;
   cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (D == 128) {   // two tiles in turn (tc_pair.cuh)
-    const int blocks = 3 * (5 + L * (6 * t->NDC + 6));   // the entries of both schedules
-    const int rest = (int)sizeof(PairMisc) + blocks * 8;
+    const int rest = (int)sizeof(PairMisc) + 3 * pair_steps(L, t->NDC) * (int)sizeof(Step);   // one tile's and two tiles'
     t->nst = (smem_optin - 1024 - rest - P_A) / A_BLOCK;
     if (t->nst > MAX_STAGES) t->nst = MAX_STAGES;
     if (t->nst < 3) return TRACKFIT_ERR_UNSUPPORTED;
@@ -954,26 +923,19 @@ int tf_tc_create(trackfit_ctx* h, const float* W) {
             make_map(&t->tm[MAP_1], t->w_1, (uint64_t)L * D, D, fp16) &&
             make_map(&t->tm[MAP_2], t->w_2, (uint64_t)L * D, D, fp16);
   if (!ok) return TRACKFIT_ERR_CUDA;
-  // ---- the per-tile block schedule, expanded once on the device
+  // ---- the schedules
   {
-    TcParams q;
-    std::memset(&q, 0, sizeof(q));
-    q.D = D;
-    q.L = L;
-    q.NDC = t->NDC;
-    q.ROWS_IN = t->ROWS_IN;
-    int* d_count = nullptr;
-    if (tf_malloc((void**)&t->sched, 4 * MAX_SCHED * sizeof(uint32_t) + 16) != cudaSuccess) return TRACKFIT_ERR_OOM;
-    d_count = reinterpret_cast<int*>(t->sched + 4 * MAX_SCHED);
-    for (int nt = 1; nt <= (D == 128 ? 2 : 1); ++nt) {
-      uint32_t* sp = t->sched + (nt - 1) * 2 * MAX_SCHED;
-      int n = 0;
-      build_schedule<<<1, 1>>>(q, nt, sp, sp + MAX_SCHED, d_count);
-      if (cudaMemcpy(&n, d_count, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return TRACKFIT_ERR_CUDA;
-      if (n < 1 || n > MAX_SCHED) return TRACKFIT_ERR_UNSUPPORTED;
-      (nt == 1 ? t->n_sched : t->n_sched2) = n;
+    std::vector<Step> steps = build_schedule(D, L, t->NDC, t->ROWS_IN, 1);
+    t->n_sched = (int)steps.size();
+    if (D == 128) {
+      const std::vector<Step> two = build_schedule(D, L, t->NDC, t->ROWS_IN, 2);
+      t->n_sched2 = (int)two.size();
+      steps.insert(steps.end(), two.begin(), two.end());
     }
-    if (D == 128 && t->n_sched + t->n_sched2 != 3 * t->n_sched) return TRACKFIT_ERR_UNSUPPORTED;
+    if (t->n_sched > MAX_SCHED || (D == 128 && (int)steps.size() > 3 * pair_steps(L, t->NDC))) return TRACKFIT_ERR_UNSUPPORTED;
+    if (tf_malloc((void**)&t->sched, steps.size() * sizeof(Step)) != cudaSuccess) return TRACKFIT_ERR_OOM;
+    if (cudaMemcpy(t->sched, steps.data(), steps.size() * sizeof(Step), cudaMemcpyHostToDevice) != cudaSuccess)
+      return TRACKFIT_ERR_CUDA;
   }
   for (auto k : {D == 128 ? tc_pair_kernel<false> : tc_forward_kernel<false>,
                  D == 128 ? tc_pair_kernel<true> : tc_forward_kernel<true>})
@@ -997,8 +959,7 @@ int tf_tc_forward(trackfit_ctx* h, const float* hits, const int32_t* n_hits, int
   p.src.slab = pk.slab;
   p.src.order = pk.order;
   p.src.n_slabs = pk.n_slabs;
-  p.sched_p = t->sched;
-  p.sched_m = t->sched + MAX_SCHED;
+  p.sched = t->sched;
   p.n_sched = t->n_sched;
   p.n_sched2 = t->n_sched2;
   p.b_e1 = t->b_e1;

@@ -19,7 +19,6 @@
 // the other tile as well (S_W_X), in place of the tile's own.
 #pragma once
 
-constexpr uint32_t S_TILE = 1u << 22, S_W_X = 1u << 23;
 enum { W_X = 4 };
 constexpr int P_XB = 0, P_HB = 32768, P_TILE = 65536, P_A = 2 * P_TILE;   // shared memory: per tile XB and HB, then the weight ring
 
@@ -27,7 +26,7 @@ constexpr int P_XB = 0, P_HB = 32768, P_TILE = 65536, P_A = 2 * P_TILE;   // sha
 // f(u, map, row, col, nk, tmem_col, bsel, bk, acc, wait, commit) as for walk_tile; u:
 // the tile; wait: a sum of W_E, W_H and W_X.
 template <class F>
-__host__ __device__ inline void walk_pair(int L, int NDC, int ROWS_IN, int nt, F&& f) {
+inline void walk_pair(int L, int NDC, int ROWS_IN, int nt, F&& f) {
   // the embedding's first product goes to the gate columns, so it can run while the
   // epilogue still pools the tiles before
   for (int u = 0; u < nt; ++u)
@@ -115,17 +114,10 @@ __global__ void __launch_bounds__(NT, 1) tc_pair_kernel(const __grid_constant__ 
     m->abort_flag = 0;
     fence_mbar_init();
   }
-  // the two schedules: producer and MMA entries of one tile, then of two
-  uint32_t* tab = reinterpret_cast<uint32_t*>(gbase + p.off_misc + sizeof(PairMisc));
+  // the steps of one tile, then those of two
+  Step* tab = reinterpret_cast<Step*>(gbase + p.off_misc + sizeof(PairMisc));
   const int n1 = p.n_sched, n2 = p.n_sched2;
-  for (int i = threadIdx.x; i < n1; i += blockDim.x) {
-    tab[i] = p.sched_p[i];
-    tab[n1 + i] = p.sched_m[i];
-  }
-  for (int i = threadIdx.x; i < n2; i += blockDim.x) {
-    tab[2 * n1 + i] = p.sched_p[2 * MAX_SCHED + i];
-    tab[2 * n1 + n2 + i] = p.sched_m[2 * MAX_SCHED + i];
-  }
+  for (int i = threadIdx.x; i < n1 + n2; i += blockDim.x) tab[i] = p.sched[i];
   if (warp == 1) {
     tmem_alloc(smem_u32(&m->tmem_base), 512);
     tmem_relinquish();
@@ -143,36 +135,40 @@ __global__ void __launch_bounds__(NT, 1) tc_pair_kernel(const __grid_constant__ 
   volatile int* abort = &m->abort_flag;
 
   if (warp == 0) {
-    // TMA producer: one 16 KB weight block per stage, in schedule order; the whole warp
-    // walks the schedule and waits, one elected lane issues
+    // TMA producer: the 16 KB weight blocks in schedule order, one ring stage each; as in
+    // the one-tile kernel, one lane's copies are let through by a predicate
     uint32_t stage = 0, phase = 0;
+    const uint32_t me = elect_one() ? 1u : 0u;
     bool ok = true;
     int issued = 0;
     for (int j = 0; j < mine && ok; j += 2) {
       const bool two = j + 1 < mine;
-      const uint32_t* t = two ? tab + 2 * n1 : tab;
+      const Step* t = two ? tab + n1 : tab;
       const int n = two ? n2 : n1;
-      for (int i = 0; i < n; ++i) {
-        const uint32_t e = t[i];
-        const bool got = mbar_wait(empty0 + 8 * stage, phase ^ 1u, abort, p.wait_ns);
-        if (!__all_sync(0xffffffffu, got)) {
-          if (lane == 0) set_abort(&m->abort_flag, p.err);
-          ok = false;
-          break;
-        }
-        if (elect_one()) {
-          mbar_arrive_expect_tx(full0 + 8 * stage, A_BLOCK);
-          tma_load_2d(ab + stage * A_BLOCK, &p.tm[e & 15u], full0 + 8 * stage, (int)((e >> 4) & 15u) * 64, (int)(e >> 8));
-        }
-        __syncwarp();
-        ++issued;
-        if (++stage == (uint32_t)p.nst) {
-          stage = 0;
-          phase ^= 1u;
+      for (int i = 0; i < n && ok; ++i) {
+        const Step e = t[i];
+        const CUtensorMap* map = &p.tm[e.prod & 15u];
+        int c0 = (int)((e.prod >> 4) & 15u) * 64;
+        const int c1 = (int)(e.prod >> 8), nb = (e.mma & S_TAIL) ? 1 : 2;
+        for (int b = 0; b < nb; ++b, c0 += 64) {
+          const uint32_t full = full0 + 8 * stage;
+          if (!mbar_wait(empty0 + 8 * stage, phase ^ 1u, abort, p.wait_ns)) {
+            set_abort(&m->abort_flag, p.err);
+            ok = false;
+            break;
+          }
+          mbar_arrive_expect_tx_if(full, A_BLOCK, me);
+          tma_load_2d_if(ab + stage * A_BLOCK, map, full, c0, c1, me);
+          ++issued;
+          if (++stage == (uint32_t)p.nst) {
+            stage = 0;
+            phase ^= 1u;
+          }
         }
       }
     }
-    if (!ok) {   // let the copies already issued land before the CTA can exit
+    __syncwarp();
+    if (*abort) {   // let the copies already issued land before the CTA can exit
       volatile int never = 0;
       for (int k = 0; k < p.nst && k < issued; ++k) {
         const int i = issued - 1 - k;
@@ -180,74 +176,85 @@ __global__ void __launch_bounds__(NT, 1) tc_pair_kernel(const __grid_constant__ 
       }
     }
   } else if (warp == 1) {
-    // MMA issuer: the whole warp walks the schedule, one elected lane issues
+    // MMA issuer: one straight line a step, as in the one-tile kernel
     uint32_t stage = 0, phase = 0;
     uint32_t e_k0 = 0, e_k1 = 0, h_k0 = 0, h_k1 = 0, a_k0 = 0, a_k1 = 0;   // hand-overs and commits so far, by tile
+    const uint32_t me = elect_one() ? 1u : 0u;
     bool ok = true;
-    const uint64_t a_desc0 = sdesc_sw128(ab, 16, 1024);
-    const uint64_t b_desc0 = sdesc_sw128(base, B_LBO, B_SBO);
+    const uint64_t a_desc = sdesc_sw128(ab, 16, 1024), b_desc = sdesc_sw128(base, B_LBO, B_SBO);
+    const uint32_t a_lo0 = desc_lo(a_desc), a_hi = desc_hi(a_desc), b_lo0 = desc_lo(b_desc), b_hi = desc_hi(b_desc);
     constexpr uint32_t BSTEP = (2 * B_SBO) >> 4;
     const uint32_t idesc = p.idesc;
-    auto wait_bar = [&](uint32_t bar, uint32_t parity) -> bool {
-      const bool got = mbar_wait(bar, parity, abort, p.wait_ns);
-      if (__all_sync(0xffffffffu, got)) return true;
-      if (lane == 0) set_abort(&m->abort_flag, p.err);
-      return false;
+    auto wait_bar = [&](uint32_t bar, uint32_t parity) {
+      if (!mbar_wait(bar, parity, abort, p.wait_ns)) {
+        set_abort(&m->abort_flag, p.err);
+        ok = false;
+      }
     };
-    auto wait_e = [&](uint32_t u) -> bool {   // tile u's k-th operand hand-over arrives on e_bar[u][k % 2]
+    auto wait_e = [&](uint32_t u) {   // tile u's k-th operand hand-over arrives on e_bar[u][k % 2]
       const uint32_t k = u ? e_k1 : e_k0;
-      if (u) ++e_k1; else ++e_k0;
-      return wait_bar(e_bar + 16 * u + 8 * (k & 1u), (k >> 1) & 1u);
-    };
-    auto wait_h = [&](uint32_t u) -> bool {
-      const uint32_t k = u ? h_k1 : h_k0;
-      if (u) ++h_k1; else ++h_k0;
-      return wait_bar(eh_bar + 8 * u, k & 1u);
+      e_k0 += u ^ 1u;
+      e_k1 += u;
+      wait_bar(e_bar + 16 * u + 8 * (k & 1u), (k >> 1) & 1u);
     };
     for (int j = 0; j < mine && ok; j += 2) {
       const bool two = j + 1 < mine;
       const int n = two ? n2 : n1;
-      const uint32_t* t = two ? tab + 2 * n1 + n2 : tab + n1;
+      const Step* t = two ? tab + n1 : tab;
+      uint32_t e = t[0].mma;
       for (int i = 0; i < n; ++i) {
-        const uint32_t e = t[i], u = (e & S_TILE) ? 1u : 0u;
-        if (e & (S_W_E | S_W_H | S_W_X)) {
-          if ((e & S_W_E) && !(ok = wait_e(u))) break;
-          if ((e & S_W_X) && !(ok = wait_e(u ^ 1u))) break;
-          if ((e & S_W_H) && !(ok = wait_h(u))) break;
+        const uint32_t en = t[i + 1 < n ? i + 1 : 0].mma, u = (e & S_TILE) ? 1u : 0u;
+        if (e & S_W_E) wait_e(u);
+        if (e & S_W_X) wait_e(u ^ 1u);
+        if (e & S_W_H) {
+          const uint32_t k = u ? h_k1 : h_k0;
+          h_k0 += u ^ 1u;
+          h_k1 += u;
+          wait_bar(eh_bar + 8 * u, k & 1u);
         }
-        if (!mbar_test_wait(full0 + 8 * stage, phase) && !(ok = wait_bar(full0 + 8 * stage, phase))) break;
-        tc_fence_after();
-        uint32_t acc_b = 0;
+        wait_bar(full0 + 8 * stage, phase);
+        if (!ok) break;
+        const uint32_t a_lo = a_lo0 + stage * (A_BLOCK >> 4), b_lo = b_lo0 + (e & 0xFFFFu);
+        const uint32_t d = tmem + ((e & S_COL) >> 16) * 128u;
+        if (e & S_TAIL) {
+          tc_fence_after();
+          umma2_f16_if<BSTEP>(d, a_lo, a_hi, b_lo, b_hi, idesc, 1u, me);
+          umma_commit_if(empty0 + 8 * stage, me);
+        } else {
+          const uint32_t s0 = stage;
+          if (++stage == (uint32_t)p.nst) {
+            stage = 0;
+            phase ^= 1u;
+          }
+          wait_bar(full0 + 8 * stage, phase);
+          if (!ok) break;
+          tc_fence_after();
+          umma4_f16_if<BSTEP>(d, a_lo, a_hi, b_lo, b_hi, idesc, e & S_ACC, me);
+          umma_commit_if(empty0 + 8 * s0, me);
+          umma4_f16_if<BSTEP>(d, a_lo0 + stage * (A_BLOCK >> 4), a_hi, b_lo + 4 * BSTEP, b_hi, idesc, 1u, me);
+          umma_commit_if(empty0 + 8 * stage, me);
+        }
         if (e & S_C_ACC) {   // tile u's k-th accumulator commit goes to acc_bar[u][k % 2]
           const uint32_t k = u ? a_k1 : a_k0;
-          acc_b = acc_bar + 16 * u + 8 * (k & 1u);
-          if (u) ++a_k1; else ++a_k0;
+          a_k0 += u ^ 1u;
+          a_k1 += u;
+          umma_commit_if(acc_bar + 16 * u + 8 * (k & 1u), me);
+        } else if (e & S_C_HB) {
+          umma_commit_if(hb_bar + 8 * u, me);
         }
-        if (elect_one()) {
-          const uint64_t ad = a_desc0 + (uint64_t)((stage * A_BLOCK) >> 4);
-          const uint64_t bd = b_desc0 + (uint64_t)((u * P_TILE + (((e >> 13) & 1u) ? P_HB : P_XB)) >> 4) +
-                              (uint64_t)(e & 0x1FFFu);
-          const uint32_t d = tmem + ((e >> 14) & 3u) * 128u, nk4 = e & S_NK4;
-          umma_f16(d, ad, bd, idesc, e & S_ACC);
-          umma_f16(d, ad + 2, bd + BSTEP, idesc, 1u);
-          umma_f16_if(d, ad + 4, bd + 2 * BSTEP, idesc, 1u, nk4);
-          umma_f16_if(d, ad + 6, bd + 3 * BSTEP, idesc, 1u, nk4);
-          umma_commit(empty0 + 8 * stage);
-          umma_commit_if(acc_b, e & S_C_ACC);
-          umma_commit_if(hb_bar + 8 * u, e & S_C_HB);
-        }
-        __syncwarp();
+        e = en;
         if (++stage == (uint32_t)p.nst) {
           stage = 0;
           phase ^= 1u;
         }
       }
     }
-    // no MMA may still run when TMEM is released
-    if (elect_one()) umma_commit(drain_bar);
     __syncwarp();
+    // no MMA may still run when TMEM is released (by the lane that issued them)
+    umma_commit_if(drain_bar, me);
     volatile int never = 0;
     mbar_wait(drain_bar, 0, &never, DRAIN_NS);
+    __syncwarp();
   } else if (warp < 2 + NE / 32) {
     // Epilogue: every step for tile 0, then for tile 1.  The warps run decoupled, as in
     // the one-tile kernel; its argument that no warp is two hand-overs ahead or two
