@@ -21,6 +21,8 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include "trackfit_internal.h"
+
 namespace tf_attn {
 
 __device__ __forceinline__ void put(float* p, float v) { *p = v; }
@@ -249,10 +251,8 @@ inline cudaError_t allow_smem(int T, int D, int NH) {
   if (sm <= 48 * 1024) return cudaSuccess;
 #define TF_ATTN_ATTR(DHV)                                                                                    \
   case DHV:                                                                                                  \
-    return T <= 32 ? cudaFuncSetAttribute(track_attention_kernel<DHV, 32, OutT>,                             \
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, sm)                   \
-                   : cudaFuncSetAttribute(track_attention_kernel<DHV, 64, OutT>,                             \
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    return T <= 32 ? tf_allow_smem(track_attention_kernel<DHV, 32, OutT>)                                    \
+                   : tf_allow_smem(track_attention_kernel<DHV, 64, OutT>);
   switch (D / NH) {
     TF_ATTN_ATTR(8)
     TF_ATTN_ATTR(16)

@@ -331,7 +331,7 @@ __global__ void __launch_bounds__(NT, 1) concat_kernel(const __grid_constant__ C
         const bool got = mbar_wait(smem_u32(&m->meta_free[b]), (uint32_t)((i >> 1) - 1) & 1u, abort, p.wait_ns);
         if (!__all_sync(0xffffffffu, got) && lane == 0) cat_abort(m, p.err);
       }
-      load_meta(p.src, nullptr, &m->meta[b], t, n_slabs, lane);
+      load_meta(p.src, nullptr, &m->meta[b], 2 * t, n_slabs, lane);
       __threadfence_block();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&m->meta_full[b]));
@@ -435,9 +435,9 @@ int tf_cat_create(trackfit_ctx* h, const float* W, tf_cat_state** out) {
   p.b_e2 = db + D;
   p.b_in = db + 2 * D;
   int64_t chunk = 1 << 20;
-  while (chunk > 1024 && (size_t)slab_bound(chunk, s.T) * SLAB * E * 2 + (size_t)chunk * 2 * H * 4 > CT_WS_BUDGET) chunk -= 1024;
+  while (chunk > 1024 && (size_t)tf_slab_bound(chunk, s.T) * SLAB * E * 2 + (size_t)chunk * 2 * H * 4 > CT_WS_BUDGET) chunk -= 1024;
   c->chunk = chunk;
-  const int64_t cap = (slab_bound(chunk, s.T) + 1) / 2 * TILE;
+  const int64_t cap = (tf_slab_bound(chunk, s.T) + 1) / 2 * TILE;
   if (st == TRACKFIT_OK) st = tf_status_from_cuda(tf_malloc(&c->pack, tf_pack_bytes(chunk)));
   if (st == TRACKFIT_OK) st = tf_status_from_cuda(tf_malloc((void**)&c->four, (size_t)cap * E * 2));
   if (st == TRACKFIT_OK) st = tf_status_from_cuda(tf_malloc((void**)&c->pool, (size_t)chunk * 2 * H * 4));
@@ -450,10 +450,9 @@ int tf_cat_create(trackfit_ctx* h, const float* W, tf_cat_state** out) {
       !tile_map(&p.tm[CM_E2], we2, D, D, fp16) || !tile_map(&p.tm[CM_IN0], w0, rows, D, fp16) ||
       !tile_map(&p.tm[CM_IN1], w1, rows, 2 * H, fp16))
     return TRACKFIT_ERR_CUDA;
-  for (auto k : {concat_kernel<false>, concat_kernel<true>})
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->smem) != cudaSuccess)
-      return TRACKFIT_ERR_CUDA;
-  if (tf_head_prepare(s.P) != cudaSuccess) return TRACKFIT_ERR_CUDA;
+  if (tf_allow_smem(concat_kernel<false>) != cudaSuccess || tf_allow_smem(concat_kernel<true>) != cudaSuccess)
+    return TRACKFIT_ERR_CUDA;
+  if (tf_head_prepare() != cudaSuccess) return TRACKFIT_ERR_CUDA;
   return TRACKFIT_OK;
 }
 

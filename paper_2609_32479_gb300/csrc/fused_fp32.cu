@@ -282,8 +282,7 @@ bool tf_fused_fp32_supported(const tf_shape& s) {
 
 cudaError_t tf_fused_fp32_prepare(const tf_shape& s) {
   for (int RM : {1, 4}) {
-    const Plan q = shape_plan(s, RM);
-    const cudaError_t e = cudaFuncSetAttribute(pick(q), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)q.smem);
+    const cudaError_t e = tf_allow_smem(pick(shape_plan(s, RM)));
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -20,7 +20,6 @@ struct HeadArgs {
   unsigned long long* err;
 };
 
-// hid lies over the normed vectors' region once they have been read
 size_t head_smem(int RM, int P) {
   return (size_t)(16 * RM * (P + 4) + 16 * RM * 132 + tf_ffma::stage_floats(8)) * 4;
 }
@@ -78,11 +77,9 @@ __global__ void __launch_bounds__(tf_ffma::NTHREADS) head_kernel(const __grid_co
 
 }  // namespace
 
-cudaError_t tf_head_prepare(int P) {
-  const cudaError_t e = cudaFuncSetAttribute(head_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)head_smem(1, P));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(head_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)head_smem(2, P));
+cudaError_t tf_head_prepare() {
+  const cudaError_t e = tf_allow_smem(head_kernel<1>);
+  return e != cudaSuccess ? e : tf_allow_smem(head_kernel<2>);
 }
 
 // 32 tracks a CTA; 16 while that leaves SMs without a CTA (a small batch is bound by

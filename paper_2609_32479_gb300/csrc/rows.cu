@@ -615,7 +615,10 @@ __global__ void pool_mean_rows_kernel(const float* __restrict__ x, const int64_t
 
 // ------------------------------------------------------------------ host side
 struct tf_rows_state {
-  tf_cat_state* cat;        // the configurations that concat.cu takes: nothing below but wait_ns is set up then
+  // the configurations that concat.cu or transformer.cu takes: nothing below but
+  // wait_ns is set up then
+  tf_cat_state* cat;
+  tf_tr_state* tr;
   int fp16;
   int nsm;
   uint16_t* w16;            // every product's weights, 16-bit, back to back
@@ -765,6 +768,7 @@ void tf_rows_destroy(trackfit_ctx* h) {
   tf_rows_state* r = h->rows;
   if (!r) return;
   tf_cat_destroy(r->cat);
+  tf_tr_destroy(r->tr);
   tf_free(r->w16);
   tf_free(r->vec);
   tf_free(r->row0);
@@ -796,6 +800,7 @@ int tf_rows_create(trackfit_ctx* h, const float* host_w) {
   r->fp16 = s.precision == TRACKFIT_FP16_PROJ;
   r->wait_ns = RG_WAIT_NS;
   if (tf_cat_supported(s)) return tf_cat_create(h, host_w, &r->cat);
+  if (tf_tr_supported(s)) return tf_tr_create(h, host_w, &r->tr);
   r->doubling = 1;
   for (int k = 0; k + 3 < TRACKFIT_MAX_FOURIER; ++k)
     if (s.scale[k + 3] != 2.0f * s.scale[k]) r->doubling = 0;
@@ -946,8 +951,7 @@ int tf_rows_create(trackfit_ctx* h, const float* host_w) {
   upd(r->e2);
   for (int l = 0; l < s.L; ++l)
     for (int k = 0; k < (attn ? 4 : 1); ++k) upd(r->lay[l][k]);
-  if (cudaFuncSetAttribute(row_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)r->smem) != cudaSuccess)
-    return TRACKFIT_ERR_CUDA;
+  if (tf_allow_smem(row_gemm_kernel) != cudaSuccess) return TRACKFIT_ERR_CUDA;
   {   // one CTA of every product must fit on an SM (registers, shared memory)
     int per_sm = 0;
     const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, row_gemm_kernel, RG_THREADS, r->smem);
@@ -957,7 +961,7 @@ int tf_rows_create(trackfit_ctx* h, const float* host_w) {
       return TRACKFIT_ERR_UNSUPPORTED;
     }
   }
-  if (tf_head_prepare(s.P) != cudaSuccess) return TRACKFIT_ERR_CUDA;
+  if (tf_head_prepare() != cudaSuccess) return TRACKFIT_ERR_CUDA;
   if (attn && (tf_attn::allow_smem<__half>(s.T, s.D, s.NH) != cudaSuccess ||
                tf_attn::allow_smem<__nv_bfloat16>(s.T, s.D, s.NH) != cudaSuccess))
     return TRACKFIT_ERR_CUDA;
@@ -1028,6 +1032,7 @@ int tf_rows_forward(trackfit_ctx* h, const float* hits, const int32_t* n_hits, i
   tf_rows_state* r = h->rows;
   const tf_shape& s = h->s;
   if (r->cat) return tf_cat_forward(h, r->cat, r->wait_ns, hits, n_hits, B, out, out_q, out_pool, st, offs);
+  if (r->tr) return tf_tr_forward(h, r->tr, r->wait_ns, hits, n_hits, B, out, out_q, out_pool, st, offs);
   for (int64_t c0 = 0; c0 < B; c0 += r->chunk) {
     const int64_t nb = B - c0 < r->chunk ? B - c0 : r->chunk;
     const float* hc = offs ? hits : hits + c0 * s.T * s.F;

@@ -521,14 +521,14 @@ __device__ __forceinline__ void scan_chain_store(const ECtx& x, float (&a)[32], 
 // the metadata buffer md), the features of its hits, and the Fourier operand
 // (the B operand of the embedding's first product) as the byte image of HB in
 // the CTA's global buffer fb, from which the epilogue copies it at tile start.
-__device__ __forceinline__ void load_meta(const TileSrc& p, uint8_t* col_tpos, TileMeta* md, int tile, int n_slabs,
-                                          int lane) {
+// The tile's slabs are s0 and, if there is one before end, s0 + 1.
+__device__ __forceinline__ void load_meta(const TileSrc& p, uint8_t* col_tpos, TileMeta* md, int s0, int end, int lane) {
   for (int c = lane; c < TILE; c += 32) md->col_flags[c] = 0;
   __syncwarp();
   int ns = 0;
   for (int hf = 0; hf < 2; ++hf) {
-    const int s = 2 * tile + hf;
-    if (s >= n_slabs) break;
+    const int s = s0 + hf;
+    if (s >= end) break;
     const int2 sl = p.slab[s];
     const int b0 = sl.x, cnt = sl.y;
     int n = 0, trk = 0;
@@ -575,9 +575,9 @@ __device__ __forceinline__ void load_meta(const TileSrc& p, uint8_t* col_tpos, T
 }
 
 template <bool FP16>
-__device__ __forceinline__ void load_tile(const TileSrc& p, LoaderScratch* m, TileMeta* md, uint8_t* fb, int tile,
-                                          int n_slabs, int lane) {
-  load_meta(p, m->col_tpos, md, tile, n_slabs, lane);
+__device__ __forceinline__ void load_tile(const TileSrc& p, LoaderScratch* m, TileMeta* md, uint8_t* fb, int s0,
+                                          int end, int lane) {
+  load_meta(p, m->col_tpos, md, s0, end, lane);
   for (int idx = lane; idx < TILE * 5; idx += 32) {
     const int col = idx / 5, f = idx - col * 5;
     float v = 0.0f;

@@ -85,7 +85,7 @@ struct TcParams {
   uint64_t wait_ns;     // limit of every bounded wait
   int hold_tile;        // test hook: CTA 0's loader holds this tile's metadata hand-over (-1: none)
   int D, L, NDC, ROWS_IN, nst;
-  uint32_t idesc;
+  uint32_t idesc, idesc_thin;   // N = 128, 64
   int off_xb, off_hb, off_a, off_misc;
   int fp16;
   float rms_eps;
@@ -525,7 +525,7 @@ __global__ void __launch_bounds__(NT, 1) tc_forward_kernel(const __grid_constant
         if (!__all_sync(0xffffffffu, got) && lane == 0) set_abort(&m->abort_flag, p.err);
         free_ph[b] ^= 1u;
       }
-      load_tile<FP16>(p.src, &m->ls, &m->meta[b], fbuf + b * EB_BYTES, t, n_slabs, lane);
+      load_tile<FP16>(p.src, &m->ls, &m->meta[b], fbuf + b * EB_BYTES, 2 * t, n_slabs, lane);
       __threadfence_block();
       __syncwarp();
       if (i == p.hold_tile && blockIdx.x == 0) {
@@ -679,7 +679,7 @@ struct tf_tc_state {
   int nsm = 0, nst = 0, NDC = 0, ROWS_IN = 0, KM = 0;
   size_t smem = 0;
   int off_xb = 0, off_hb = 0, off_a = 0, off_misc = 0;
-  uint32_t idesc = 0;
+  uint32_t idesc = 0, idesc_thin = 0;
   void* dev = nullptr;  // one allocation for all weights
   uint16_t *w_e1 = nullptr, *w_e2 = nullptr, *w_in = nullptr, *w_m = nullptr, *w_1 = nullptr, *w_2 = nullptr;
   float *b_e1 = nullptr, *b_e2 = nullptr, *g = nullptr, *b_in = nullptr, *b_m = nullptr, *b_1 = nullptr,
@@ -813,6 +813,7 @@ int tf_tc_create(trackfit_ctx* h, const float* W) {
   t->KM = t->NDC * 128;
   const bool fp16 = s.precision == TRACKFIT_FP16_PROJ;
   t->idesc = idesc_f16(128, 128, fp16 ? 0u : 1u, false, true);
+  t->idesc_thin = idesc_f16(128, 64, fp16 ? 0u : 1u, false, true);
   int dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&t->nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -937,11 +938,13 @@ int tf_tc_create(trackfit_ctx* h, const float* W) {
     if (cudaMemcpy(t->sched, steps.data(), steps.size() * sizeof(Step), cudaMemcpyHostToDevice) != cudaSuccess)
       return TRACKFIT_ERR_CUDA;
   }
-  for (auto k : {D == 128 ? tc_pair_kernel<false> : tc_forward_kernel<false>,
-                 D == 128 ? tc_pair_kernel<true> : tc_forward_kernel<true>})
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)t->smem) != cudaSuccess)
-      return TRACKFIT_ERR_CUDA;
-  if (tf_head_prepare(s.P) != cudaSuccess)
+  if (tf_allow_smem(tc_forward_kernel<false>) != cudaSuccess || tf_allow_smem(tc_forward_kernel<true>) != cudaSuccess ||
+      tf_allow_smem(tc_pair_kernel<false, false>) != cudaSuccess ||
+      tf_allow_smem(tc_pair_kernel<true, false>) != cudaSuccess ||
+      tf_allow_smem(tc_pair_kernel<false, true>) != cudaSuccess ||
+      tf_allow_smem(tc_pair_kernel<true, true>) != cudaSuccess)
+    return TRACKFIT_ERR_CUDA;
+  if (tf_head_prepare() != cudaSuccess)
     return TRACKFIT_ERR_CUDA;
   return TRACKFIT_OK;
 }
@@ -979,6 +982,7 @@ int tf_tc_forward(trackfit_ctx* h, const float* hits, const int32_t* n_hits, int
   p.ROWS_IN = t->ROWS_IN;
   p.nst = t->nst;
   p.idesc = t->idesc;
+  p.idesc_thin = t->idesc_thin;
   p.off_xb = t->off_xb;
   p.off_hb = t->off_hb;
   p.off_a = t->off_a;
@@ -1006,9 +1010,12 @@ int tf_tc_forward(trackfit_ctx* h, const float* hits, const int32_t* n_hits, int
     p.src.n_hits = n_hits + c0;
     p.pool = out_pool ? out_pool + c0 * s.P : t->pool;
     tf_prof_begin(h, st);
-    const auto kernel = s.D == 128 ? (p.fp16 ? tc_pair_kernel<true> : tc_pair_kernel<false>)
+    // as many CTAs as slabs there can be: one-slab tiles (d_model 128)
+    const bool thin = s.D == 128 && tf_slab_bound(nb, s.T) <= t->nsm;
+    const auto kernel = s.D == 128 ? (p.fp16 ? (thin ? tc_pair_kernel<true, true> : tc_pair_kernel<true, false>)
+                                             : (thin ? tc_pair_kernel<false, true> : tc_pair_kernel<false, false>))
                                    : (p.fp16 ? tc_forward_kernel<true> : tc_forward_kernel<false>);
-    kernel<<<t->nsm, NT, t->smem, st>>>(p);
+    kernel<<<t->nsm, thin ? PAIR_NT<true> : NT, t->smem, st>>>(p);
     tf_prof_end(h, st);
     if (tf_head(s, h->off, h->d_w, p.pool, p.src.n_hits, nb, t->nsm, out + c0 * 5, out_q ? out_q + c0 * s.Q : nullptr,
                 out_pool ? p.pool : nullptr, h->d_err, st) != cudaSuccess)

@@ -81,8 +81,17 @@ struct PairMisc {
   alignas(16) float rinv[NE / 32][32];
 };
 
-template <bool FP16>
-__global__ void __launch_bounds__(NT, 1) tc_pair_kernel(const __grid_constant__ TcParams p) {
+// THIN: a tile is one slab, with half the columns and half the epilogue warps.  While
+// every slab can have a CTA of its own the batch's time is one tile's chain of steps,
+// and that is shorter then.
+template <bool THIN>
+constexpr int PAIR_EPI = THIN ? NE / 64 : NE / 32;   // epilogue warps
+template <bool THIN>
+constexpr int PAIR_NT = 32 * (PAIR_EPI<THIN> + 3);
+
+template <bool FP16, bool THIN>
+__global__ void __launch_bounds__(PAIR_NT<THIN>, 1) tc_pair_kernel(const __grid_constant__ TcParams p) {
+  constexpr int EW = PAIR_EPI<THIN>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -102,13 +111,13 @@ __global__ void __launch_bounds__(NT, 1) tc_pair_kernel(const __grid_constant__ 
     }
     for (int i = 0; i < 4; ++i) {
       mbar_init(acc_bar + 8 * i, 1);
-      mbar_init(e_bar + 8 * i, NE / 32);   // one arrival per epilogue warp
+      mbar_init(e_bar + 8 * i, EW);   // one arrival per epilogue warp
       mbar_init(smem_u32(&m->meta_full[i]), 1);
-      mbar_init(smem_u32(&m->meta_free[i]), NE / 32);
+      mbar_init(smem_u32(&m->meta_free[i]), EW);
     }
     for (int u = 0; u < 2; ++u) {
       mbar_init(hb_bar + 8 * u, 1);
-      mbar_init(eh_bar + 8 * u, NE / 32);
+      mbar_init(eh_bar + 8 * u, EW);
     }
     mbar_init(drain_bar, 1);
     m->abort_flag = 0;
@@ -129,7 +138,7 @@ __global__ void __launch_bounds__(NT, 1) tc_pair_kernel(const __grid_constant__ 
   tc_fence_after();
   const uint32_t tmem = m->tmem_base;
   const int n_slabs = *p.src.n_slabs;
-  const int n_tiles = (n_slabs + 1) >> 1;
+  const int n_tiles = THIN ? n_slabs : (n_slabs + 1) >> 1;
   int mine = 0;   // this CTA's tiles: blockIdx.x + j gridDim.x
   if ((int)blockIdx.x < n_tiles) mine = (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;
   volatile int* abort = &m->abort_flag;
@@ -184,7 +193,7 @@ __global__ void __launch_bounds__(NT, 1) tc_pair_kernel(const __grid_constant__ 
     const uint64_t a_desc = sdesc_sw128(ab, 16, 1024), b_desc = sdesc_sw128(base, B_LBO, B_SBO);
     const uint32_t a_lo0 = desc_lo(a_desc), a_hi = desc_hi(a_desc), b_lo0 = desc_lo(b_desc), b_hi = desc_hi(b_desc);
     constexpr uint32_t BSTEP = (2 * B_SBO) >> 4;
-    const uint32_t idesc = p.idesc;
+    const uint32_t idesc = THIN ? p.idesc_thin : p.idesc;   // N = 64, 128
     auto wait_bar = [&](uint32_t bar, uint32_t parity) {
       if (!mbar_wait(bar, parity, abort, p.wait_ns)) {
         set_abort(&m->abort_flag, p.err);
@@ -255,7 +264,7 @@ __global__ void __launch_bounds__(NT, 1) tc_pair_kernel(const __grid_constant__ 
     volatile int never = 0;
     mbar_wait(drain_bar, 0, &never, DRAIN_NS);
     __syncwarp();
-  } else if (warp < 2 + NE / 32) {
+  } else if (warp < 2 + EW) {
     // Epilogue: every step for tile 0, then for tile 1.  The warps run decoupled, as in
     // the one-tile kernel; its argument that no warp is two hand-overs ahead or two
     // commits behind holds for each tile's own barriers.  A failed wait sets the abort
@@ -314,18 +323,25 @@ __global__ void __launch_bounds__(NT, 1) tc_pair_kernel(const __grid_constant__ 
       wait_on(hb_bar + 8 * u, k & 1u);
     };
     // the Fourier operand of tile u of a pair: the loads need the loader's hand-over,
-    // the stores need the tile's HB and XB free
+    // the stores need the tile's HB and XB free.
     const uint8_t* fbuf = p.fbuf + (size_t)blockIdx.x * 4 * EB_BYTES;
+    // a thread's r-th 16-byte chunk of the operand (THIN: the first 64 columns, the first of
+    // each two 1 KB atoms)
+    auto chunk = [&](int r) -> uint32_t {
+      const uint32_t i = (uint32_t)(r * EW * 32 + x.te);
+      return THIN ? (i >> 6) * (uint32_t)B_SBO + (i & 63u) * 16u : i * 16u;
+    };
     auto fetch = [&](int pr, int u, uint4 (&v)[5]) {
       const int b = 2 * (pr & 1) + u;
       wait_on(smem_u32(&m->meta_full[b]), (uint32_t)(pr >> 1) & 1u);
-      fourier_fetch(x, fbuf + b * EB_BYTES, v);
+#pragma unroll
+      for (int r = 0; r < 5; ++r) v[r] = __ldcg(reinterpret_cast<const uint4*>(fbuf + b * EB_BYTES + chunk(r)));
     };
     auto put = [&](int u, const uint4 (&v)[5]) {
       const uint32_t hb = base + P_HB + u * P_TILE, xb = base + P_XB + u * P_TILE;
 #pragma unroll
-      for (int r = 0; r < 4; ++r) st_shared_v4(hb + 16 * (r * NE + x.te), v[r].x, v[r].y, v[r].z, v[r].w);
-      st_shared_v4(xb + 16 * x.te, v[4].x, v[4].y, v[4].z, v[4].w);
+      for (int r = 0; r < 4; ++r) st_shared_v4(hb + chunk(r), v[r].x, v[r].y, v[r].z, v[r].w);
+      st_shared_v4(xb + chunk(4) - 128 * 256, v[4].x, v[4].y, v[4].z, v[4].w);   // k-rows 128-159
       signal_e(u, true);
     };
     for (int u = 0; u < 2 && u < mine; ++u) {
@@ -421,8 +437,8 @@ __global__ void __launch_bounds__(NT, 1) tc_pair_kernel(const __grid_constant__ 
         const bool got = mbar_wait(smem_u32(&m->meta_free[b]), (uint32_t)((pr >> 1) - 1) & 1u, abort, p.wait_ns);
         if (!__all_sync(0xffffffffu, got) && lane == 0) set_abort(&m->abort_flag, p.err);
       }
-      load_tile<FP16>(p.src, &m->ls, &m->meta[b], fbuf + b * EB_BYTES, (int)blockIdx.x + j * (int)gridDim.x, n_slabs,
-                      lane);
+      const int t = (int)blockIdx.x + j * (int)gridDim.x;
+      load_tile<FP16>(p.src, &m->ls, &m->meta[b], fbuf + b * EB_BYTES, THIN ? t : 2 * t, THIN ? t + 1 : n_slabs, lane);
       __threadfence_block();
       __syncwarp();
       if (j == p.hold_tile && blockIdx.x == 0) {   // test hook, as in the one-tile kernel

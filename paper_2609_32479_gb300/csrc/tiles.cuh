@@ -118,12 +118,4 @@ inline uint16_t to_16(float f, bool fp16) {
   return *reinterpret_cast<const uint16_t*>(&v);
 }
 
-// Slabs that n tracks of up to T hits take at most: a slab holds at least 64 / T
-// full-length tracks (or 16 tracks), and each of a segment's 256 tracks' last slab may be
-// part-filled.
-inline int64_t slab_bound(int64_t n, int T) {
-  const int64_t per = SLAB / T < TF_SLAB_TRACKS ? SLAB / T : TF_SLAB_TRACKS;
-  return (n + per - 1) / per + n / 256 + 2;
-}
-
 }  // namespace

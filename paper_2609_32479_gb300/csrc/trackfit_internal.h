@@ -100,6 +100,20 @@ int tf_simt_forward(trackfit_ctx* h, const float* hits, const int32_t* n_hits, i
 int tf_simt_debug_scan(const float* a, const float* b, const float* x, const int32_t* n_hits,
                        int64_t B, int T, int C, float* hf, float* hb, cudaStream_t st);
 
+// Let launches of kernel take all the dynamic shared memory that a block can have.  The
+// limit belongs to the kernel, not to a handle: set to one handle's need it would keep
+// another handle's larger launch from running.
+template <class K>
+inline cudaError_t tf_allow_smem(K* kernel) {
+  int dev = 0, optin = 0;
+  cudaFuncAttributes a;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, kernel);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)a.sharedSizeBytes);
+}
+
 // plan.cu: tracks packed whole into slabs.  Slab i holds the tracks order[slab[i].x]
 // .. order[slab[i].x + slab[i].y - 1]; n_slabs[0] slabs for up to cap tracks.
 struct tf_pack {
@@ -110,6 +124,13 @@ struct tf_pack {
 };
 cudaError_t tf_plan(const int32_t* n_hits, int64_t B, int T, int nsm, int32_t* order, int2* slab, int32_t* n_slabs,
                     cudaStream_t st);
+// Slabs that n tracks of up to T hits take at most: a slab holds at least 64 / T
+// full-length tracks (or 16 tracks), and the last slab of each segment (256 tracks or
+// more) may be part-filled.
+inline int64_t tf_slab_bound(int64_t n, int T) {
+  const int64_t per = TF_SLAB / T < TF_SLAB_TRACKS ? TF_SLAB / T : TF_SLAB_TRACKS;
+  return (n + per - 1) / per + n / 256 + 2;
+}
 // The three arrays of tf_pack in one buffer of tf_pack_bytes(cap) bytes.
 inline size_t tf_pack_bytes(int64_t cap) { return 256 + (size_t)cap * 12; }
 inline tf_pack tf_pack_in(void* buf, int64_t cap) {
@@ -119,7 +140,7 @@ inline tf_pack tf_pack_in(void* buf, int64_t cap) {
 }
 
 // head.cu
-cudaError_t tf_head_prepare(int P);   // shared memory of the launches below
+cudaError_t tf_head_prepare();   // shared memory of the launches below
 cudaError_t tf_head(const tf_shape& s, const tf_blob_off& o, const float* W, const float* pooled,
                     const int32_t* n_hits, int64_t B, int nsm, float* out, float* out_q, float* out_pool,
                     unsigned long long* err, cudaStream_t st);
@@ -149,6 +170,14 @@ int tf_cat_create(trackfit_ctx* h, const float* host_w, tf_cat_state** out);
 void tf_cat_destroy(tf_cat_state* c);
 int tf_cat_forward(trackfit_ctx* h, tf_cat_state* c, uint64_t wait_ns, const float* hits, const int32_t* n_hits,
                    int64_t B, float* out, float* out_q, float* out_pool, cudaStream_t st, const int64_t* offs);
+
+// transformer.cu: the Transformer in one kernel, likewise
+struct tf_tr_state;
+bool tf_tr_supported(const tf_shape& s);
+int tf_tr_create(trackfit_ctx* h, const float* host_w, tf_tr_state** out);
+void tf_tr_destroy(tf_tr_state* c);
+int tf_tr_forward(trackfit_ctx* h, tf_tr_state* c, uint64_t wait_ns, const float* hits, const int32_t* n_hits,
+                  int64_t B, float* out, float* out_q, float* out_pool, cudaStream_t st, const int64_t* offs);
 
 // rows.cu
 bool tf_rows_supported(const tf_shape& s);

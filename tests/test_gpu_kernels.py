@@ -1,6 +1,8 @@
 """Sizes where a kernel's split can go wrong, against the oracle: the fused fp32
 encoder (each column tiling, 16- and 64-row CTAs, runs of tracks and packed slabs),
-the head's two CTA sizes, and the seed's foot points on strongly curved tracks."""
+the tile kernels of the paper's model and the Transformer (one slab to several tiles a
+CTA, tracks of 1 to 64 hits, partial Fourier chunks, head and MLP widths), the head's two
+CTA sizes, and the seed's foot points on strongly curved tracks."""
 import dataclasses
 
 import numpy as np
@@ -63,6 +65,61 @@ def test_fused_fp32_encoder_shapes(T, D, hits, n, pool):
     assert track_errors(got[ok], ref[ok]).max() <= FP32_TOL
 
 
+# (topology, features, layers, heads, MLP width, max_hits, tracks)
+TILE_SHAPES = [
+    (W.TOPOLOGY_CONCAT, 15, 1, 0, 192, 24, 1), (W.TOPOLOGY_CONCAT, 15, 2, 0, 192, 64, 70),
+    (W.TOPOLOGY_CONCAT, 16, 2, 0, 192, 3, 200), (W.TOPOLOGY_CONCAT, 1, 2, 0, 192, 33, 120),
+    (W.TOPOLOGY_CONCAT, 5, 2, 0, 192, 12, 4000),
+    (W.TOPOLOGY_ATTENTION, 15, 1, 4, 288, 24, 1), (W.TOPOLOGY_ATTENTION, 15, 3, 4, 288, 64, 70),
+    (W.TOPOLOGY_ATTENTION, 16, 2, 8, 320, 32, 150), (W.TOPOLOGY_ATTENTION, 5, 2, 8, 16, 7, 200),
+    (W.TOPOLOGY_ATTENTION, 1, 2, 4, 144, 40, 120), (W.TOPOLOGY_ATTENTION, 5, 2, 4, 208, 12, 4000)]
+
+
+def tile_case(topo, F, L, heads, H, hits, n):
+    pool = W.POOL_ENDPOINTS if topo == W.TOPOLOGY_CONCAT else W.POOL_MEAN
+    m = W.ModelConfig(max_hits=hits, d_model=128, d_hidden=H, n_layers=L, precision=W.PRECISION_FP16, pool=pool,
+                      topology=topo, n_heads=heads or 4, n_features=F, feat_min=W.PAPER_FEAT_MIN[:F] + (0.0,) * (F - 15),
+                      feat_max=W.PAPER_FEAT_MAX[:F] + (1.0,) * (F - 15))
+    rng = np.random.default_rng(n)
+    lo, hi = np.asarray(m.feat_min), np.asarray(m.feat_max)
+    h = (lo + (hi - lo) * rng.random((n, hits, F))).astype(np.float32)
+    return m, h, rng.integers(1, hits + 1, n).astype(np.int32)
+
+
+@pytest.mark.parametrize("shape", TILE_SHAPES)
+def test_tile_kernel_shapes(T, shape):
+    m, h, nh = tile_case(*shape)
+    blob = W.gen_weights(m, 2)
+    bad = len(nh) // 2 if len(nh) > 8 else None
+    if bad:
+        nh[bad] = 0
+    got, (status, n_bad) = forward(T, m, blob, h, nh)
+    few = slice(0, len(nh) if len(nh) <= 200 else 200)
+    ref = O.forward(dataclasses.asdict(m), blob, h[few], nh[few])
+    assert n_bad == (1 if bad else 0) and status == (T.ERR_BAD_HITS if bad else T.OK)
+    ok = ~np.isnan(ref[:, 0])
+    np.testing.assert_array_equal(np.isnan(got[few]), np.isnan(ref))
+    if len(nh) > 1:
+        assert track_errors(got[few][ok], ref[ok]).max() <= FP16_TOL
+    else:   # one track has no column RMS to measure by: relative to its largest parameter
+        assert np.abs(got - ref).max() <= FP16_TOL * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("topo", [W.TOPOLOGY_CONCAT, W.TOPOLOGY_ATTENTION])
+def test_a_track_with_infinite_hits_leaves_the_others_alone(T, topo):
+    """Tracks share tiles: one whose valid hits hold infinities or NaN spoils its own row
+    only, bit for bit."""
+    m, h, nh = tile_case(topo, 5, 2, 4, 192 if topo == W.TOPOLOGY_CONCAT else 288, 12, 300)
+    blob = W.gen_weights(m, 2)
+    want, _ = forward(T, m, blob, h, nh)
+    h[17, : nh[17]] = np.inf
+    h[140, 0, 2] = np.nan
+    got, _ = forward(T, m, blob, h, nh)
+    assert not np.isfinite(got[[17, 140]]).any()
+    others = np.setdiff1d(np.arange(300), [17, 140])
+    np.testing.assert_array_equal(got[others], want[others])
+
+
 @pytest.mark.parametrize("n", [1, 16, 17, 4865])
 def test_head_cta_sizes(T, n):
     """16 tracks a CTA up to 32 an SM, 32 above: the paper's 384-wide readout against
@@ -101,3 +158,35 @@ def test_seed_foot_points(T, n, pt):
     assert near.mean() > 0.8
     d = np.abs(fv - rv)[near]
     assert np.max(d[:, :2]) < 2e-6 and np.max(d[:, 2] / np.maximum(np.abs(rv[near, 2]), 1.0)) < 1e-6
+
+
+@pytest.mark.parametrize("n,hits", [(1, 24), (2, 64), (101, 24), (300, 24), (305, 24), (149, 64), (160, 64)])
+def test_one_slab_tiles(T, n, hits):
+    """Batches whose slabs each get a CTA run in tiles of one slab, larger ones in pairs of
+    two-slab tiles: each track's result is the same as in a large batch."""
+    m = W.ModelConfig(max_hits=hits, d_model=128, d_hidden=192, n_layers=2, precision=W.PRECISION_BF16)
+    blob = W.gen_weights(m, 2)
+    h, nh = ragged(m, 2000)
+    got, _ = forward(T, m, blob, h[:n], nh[:n])
+    want, _ = forward(T, m, blob, h, nh)
+    np.testing.assert_array_equal(got, want[:n])
+
+
+def test_handles_of_different_sizes_stay_usable(T):
+    """A kernel's shared memory limit is not lowered by a later, smaller handle."""
+    dev = torch.device("cuda:0")
+    open_ = []
+    for D, prec, topo in ((256, W.PRECISION_BF16, W.TOPOLOGY_MERGE), (128, W.PRECISION_BF16, W.TOPOLOGY_MERGE),
+                          (112, W.PRECISION_FP32, W.TOPOLOGY_MERGE), (16, W.PRECISION_FP32, W.TOPOLOGY_MERGE),
+                          (256, W.PRECISION_FP16, W.TOPOLOGY_CONCAT), (64, W.PRECISION_FP16, W.TOPOLOGY_CONCAT)):
+        m = W.ModelConfig(max_hits=16, d_model=D, d_hidden=3 * D // 2, n_layers=1, precision=prec, topology=topo)
+        open_.append((m, T.Trackfit(m, W.gen_weights(m, 2))))
+    h, nh = ragged(open_[0][0], 40)
+    for m, tf in open_:
+        out = torch.full((40, 5), -7.0, device=dev)
+        tf.forward(torch.from_numpy(h).to(dev), torch.from_numpy(nh).to(dev), out)
+        torch.cuda.synchronize()
+        assert tf.device_errors() == (T.OK, 0)
+        ref = O.forward(dataclasses.asdict(m), W.gen_weights(m, 2), h, nh)
+        assert track_errors(out.cpu().numpy(), ref).max() <= 2e-2   # bf16 among them: finds a wrong track
+        tf.close()
