@@ -13,9 +13,10 @@ namespace {
 // packing of a segment depends on its hit counts alone; where its slabs lie among
 // those of the other segments does not, and neither matters to a track's results.
 //
-// It is bound by the latency of the first warp's steps (about three a slab).  One
-// lane walking a table of counts took 57 us for 101 tracks and 531 us for segments
-// of 1,024.
+// It is bound by the latency of the first warp's steps (about three a slab), so their
+// state is in registers: with the counts in shared memory and an integer division a step
+// took 400 cycles (98 us for 256 tracks of 64 hits, 31 us for 997 of 12.5), and one lane
+// walking a table of counts took 57 us for 101 tracks, 531 us for segments of 1,024.
 template <int SEG>
 __global__ void __launch_bounds__(SEG) plan_kernel(const int32_t* __restrict__ n_hits, int64_t B, int T,
                                                    int32_t* __restrict__ order, int2* __restrict__ slab,
@@ -65,44 +66,55 @@ __global__ void __launch_bounds__(SEG) plan_kernel(const int32_t* __restrict__ n
   if (len >= 0) items[pos[len] + hist[warp][len] + rank] = (int16_t)tid;
   __syncthreads();
   if (warp != 0) return;
-  uint64_t left = 0;   // bit l - 1: tracks of l hits remain
-#pragma unroll
-  for (int h = 0; h < 2; ++h)
-    left |= (uint64_t)__ballot_sync(0xffffffffu, cnt[32 * h + lane + 1] > 0) << (32 * h);
-  int o = 0, ns = 0, cap = TF_SLAB, ntr = 0, bad = cnt[0];
+  // Lane i keeps, for the lengths i + 1 and i + 33: tracks left and where the next of them
+  // is in items (packed), and 1 / length in 16 fractional bits.  A step's chain of
+  // dependent operations is then a few integer instructions and two shuffles.
+  uint32_t lo = (uint32_t)cnt[lane + 1] | ((uint32_t)pos[lane + 1] << 16);
+  uint32_t hi = (uint32_t)cnt[lane + 33] | ((uint32_t)pos[lane + 33] << 16);
+  const uint32_t inv_lo = 65536u / (lane + 1) + 1u, inv_hi = 65536u / (lane + 33) + 1u;   // exact up to 64
+  uint64_t left = (uint64_t)__ballot_sync(0xffffffffu, (lo & 0xffffu) != 0) |
+                  (uint64_t)__ballot_sync(0xffffffffu, (hi & 0xffffu) != 0) << 32;   // bit l - 1: tracks of l hits remain
+  int o = 0, ns = 0, cap = TF_SLAB, ntr = 0;
   if (lane == 0) first[0] = 0;
-  while (left || bad) {
-    const uint64_t fits = cap == TF_SLAB ? left : left & ((1ull << cap) - 1ull);
-    int l = 0, k = 0;
-    if (ntr < TF_SLAB_TRACKS) {
-      if (fits) {
-        l = 64 - __clzll((long long)fits);
-        const int c = cnt[l];
-        k = min(min(c, cap / l), TF_SLAB_TRACKS - ntr);
-        if (k == c) left &= ~(1ull << (l - 1));
-      } else if (!left) {
-        k = min(bad, TF_SLAB_TRACKS - ntr);
-        bad -= k;
-      }
-    }
-    if (k == 0) {   // the slab is full
+  while (left) {
+    uint64_t fits = cap == TF_SLAB ? left : left & ((1ull << cap) - 1ull);
+    if (fits == 0 || ntr == TF_SLAB_TRACKS) {   // the slab is full
       ++ns;
       if (lane == 0) first[ns] = (int16_t)o;
       cap = TF_SLAB;
       ntr = 0;
-      continue;
+      fits = left;
     }
-    const int at = pos[l];
+    const int b = 63 - __clzll((long long)fits), l = b + 1;
+    const uint32_t cp = __shfl_sync(0xffffffffu, b < 32 ? lo : hi, b & 31);
+    const uint32_t inv = __shfl_sync(0xffffffffu, b < 32 ? inv_lo : inv_hi, b & 31);
+    const int c = (int)(cp & 0xffffu), at = (int)(cp >> 16);
+    const int k = min(min(c, (int)(((uint32_t)cap * inv) >> 16)), TF_SLAB_TRACKS - ntr);
+    if (k == c) left &= ~(1ull << b);
+    if (lane == (b & 31)) {   // k tracks fewer, the next one k further
+      const uint32_t d = ((uint32_t)k << 16) - (uint32_t)k;
+      if (b < 32)
+        lo += d;
+      else
+        hi += d;
+    }
     if (lane < k) order[b0 + o + lane] = (int32_t)(b0 + items[at + lane]);
-    __syncwarp();
-    if (lane == 0) {
-      pos[l] = (int16_t)(at + k);
-      cnt[l] = (int16_t)(cnt[l] - k);
-    }
-    __syncwarp();
     o += k;
     ntr += k;
     cap -= k * l;
+  }
+  for (int bad = cnt[0], at = 0; bad > 0;) {   // tracks with an invalid hit count
+    if (ntr == TF_SLAB_TRACKS) {
+      ++ns;
+      if (lane == 0) first[ns] = (int16_t)o;
+      ntr = 0;
+    }
+    const int k = min(bad, TF_SLAB_TRACKS - ntr);
+    if (lane < k) order[b0 + o + lane] = (int32_t)(b0 + items[at + lane]);
+    at += k;
+    o += k;
+    ntr += k;
+    bad -= k;
   }
   ++ns;   // the last slab (a segment has at least one track)
   if (lane == 0) first[ns] = (int16_t)o;
@@ -118,13 +130,18 @@ __global__ void __launch_bounds__(SEG) plan_kernel(const int32_t* __restrict__ n
 
 // Segments of 1,024 tracks leave one slab in 200 part-filled; below one such
 // segment for each SM the plan's own latency counts for more than the fill, and
-// segments of 256 take a quarter of the steps.
+// segments of 256 take a quarter of the steps.  Up to 2,048 tracks the tiles hardly fill
+// the chip once, so the fill counts for nothing: segments of 64.  With the state in
+// registers, a whole call of 101 tracks 121 -> 115 us (d_model 128) and 106 -> 84 us (997
+// tracks of the paper's model); 4,096 tracks of 64 hits 1,160 -> 1,129 us.
 cudaError_t tf_plan(const int32_t* n_hits, int64_t B, int T, int nsm, int32_t* order, int2* slab, int32_t* n_slabs,
                     cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(n_slabs, 0, sizeof(int32_t), st);
   if (e != cudaSuccess) return e;
   if (B >= (int64_t)1024 * nsm)
     plan_kernel<1024><<<(unsigned)((B + 1023) / 1024), 1024, 0, st>>>(n_hits, B, T, order, slab, n_slabs);
+  else if (B <= 2048)
+    plan_kernel<64><<<(unsigned)((B + 63) / 64), 64, 0, st>>>(n_hits, B, T, order, slab, n_slabs);
   else
     plan_kernel<256><<<(unsigned)((B + 255) / 256), 256, 0, st>>>(n_hits, B, T, order, slab, n_slabs);
   return cudaPeekAtLastError();

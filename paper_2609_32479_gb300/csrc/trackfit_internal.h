@@ -125,11 +125,12 @@ struct tf_pack {
 cudaError_t tf_plan(const int32_t* n_hits, int64_t B, int T, int nsm, int32_t* order, int2* slab, int32_t* n_slabs,
                     cudaStream_t st);
 // Slabs that n tracks of up to T hits take at most: a slab holds at least 64 / T
-// full-length tracks (or 16 tracks), and the last slab of each segment (256 tracks or
-// more) may be part-filled.
+// full-length tracks (or 16 tracks), and the last slab of each segment (64 tracks or
+// more, 256 or more above 2,048 tracks) may be part-filled.  It never falls as n grows:
+// workspaces are sized by it once and hold every smaller batch.
 inline int64_t tf_slab_bound(int64_t n, int T) {
   const int64_t per = TF_SLAB / T < TF_SLAB_TRACKS ? TF_SLAB / T : TF_SLAB_TRACKS;
-  return (n + per - 1) / per + n / 256 + 2;
+  return (n + per - 1) / per + (n <= 2048 ? n / 64 : n / 256 + 32) + 2;
 }
 // The three arrays of tf_pack in one buffer of tf_pack_bytes(cap) bytes.
 inline size_t tf_pack_bytes(int64_t cap) { return 256 + (size_t)cap * 12; }

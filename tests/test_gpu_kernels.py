@@ -190,3 +190,18 @@ def test_handles_of_different_sizes_stay_usable(T):
         ref = O.forward(dataclasses.asdict(m), W.gen_weights(m, 2), h, nh)
         assert track_errors(out.cpu().numpy(), ref).max() <= 2e-2   # bf16 among them: finds a wrong track
         tf.close()
+
+
+@pytest.mark.parametrize("n", [63, 64, 65, 2047, 2048, 2049])
+@pytest.mark.parametrize("hits", [4, 24])
+def test_packing_segments_do_not_matter_to_a_track(T, n, hits):
+    """Segments of 64 tracks up to 2,048, of 256 above: a track's result is the same bits in
+    either, with a track of an invalid hit count among them."""
+    m = W.ModelConfig(max_hits=hits, d_model=128, d_hidden=192, n_layers=1, precision=W.PRECISION_BF16)
+    blob = W.gen_weights(m, 2)
+    h, nh = ragged(m, 2500)
+    nh[17] = 0
+    want, _ = forward(T, m, blob, h, nh)
+    got, (_, n_bad) = forward(T, m, blob, h[:n], nh[:n])
+    assert n_bad == 1
+    np.testing.assert_array_equal(got, want[:n])
