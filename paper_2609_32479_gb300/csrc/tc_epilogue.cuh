@@ -574,10 +574,8 @@ __device__ __forceinline__ void load_meta(const TileSrc& p, uint8_t* col_tpos, T
   __syncwarp();
 }
 
-template <bool FP16>
-__device__ __forceinline__ void load_tile(const TileSrc& p, LoaderScratch* m, TileMeta* md, uint8_t* fb, int s0,
-                                          int end, int lane) {
-  load_meta(p, m->col_tpos, md, s0, end, lane);
+// The features of the tile's hits.
+__device__ __forceinline__ void load_hits(const TileSrc& p, LoaderScratch* m, const TileMeta* md, int lane) {
   for (int idx = lane; idx < TILE * 5; idx += 32) {
     const int col = idx / 5, f = idx - col * 5;
     float v = 0.0f;
@@ -589,6 +587,13 @@ __device__ __forceinline__ void load_tile(const TileSrc& p, LoaderScratch* m, Ti
     m->hs[col][f] = v;
   }
   __syncwarp();
+}
+
+// The Fourier operand of the tile's first 8 groups columns, the work items first, first +
+// stride, ..: store(k-row, group of 8 columns, 16-byte chunk).
+template <bool FP16, class Store>
+__device__ __forceinline__ void fourier_operand(const TileSrc& p, const LoaderScratch* m, const TileMeta* md, int groups,
+                                                int first, int stride, Store&& store) {
   // u = (v - min) / (max - min) and the argument s_k * u as unevaluated sums of
   // two floats (error-free TwoSum / TwoProduct with fma), reduced modulo 2
   // exactly, so sin(pi s_k u) carries only the final fp32 rounding.
@@ -604,8 +609,7 @@ __device__ __forceinline__ void load_tile(const TileSrc& p, LoaderScratch* m, Ti
     return (xh - 2.0f * rintf(0.5f * xh)) + xl;
   };
   auto put = [&](int row, int g, const float (&v)[8]) {
-    *reinterpret_cast<uint4*>(fb + bchunk(row, g)) =
-        make_uint4(pack2<FP16>(v[0], v[1]), pack2<FP16>(v[2], v[3]), pack2<FP16>(v[4], v[5]), pack2<FP16>(v[6], v[7]));
+    store(row, g, make_uint4(pack2<FP16>(v[0], v[1]), pack2<FP16>(v[2], v[3]), pack2<FP16>(v[4], v[5]), pack2<FP16>(v[6], v[7])));
   };
   // one work item = 8 columns of one feature and one evaluated scale, stored as
   // 16-byte chunks of the operand.  With s_{k+3} = 2 s_k, sin/cos are evaluated
@@ -613,8 +617,8 @@ __device__ __forceinline__ void load_tile(const TileSrc& p, LoaderScratch* m, Ti
   // the double angle identities (2 s c, (c - s)(c + s)), so no value is more than
   // one doubling (a few ulp) from an evaluated one.
   const int n_eval = p.scale_doubling ? 9 : 16;
-  for (int it = lane; it < (TILE / 8) * 5 * n_eval; it += 32) {
-    const int g = it % (TILE / 8), fk = it / (TILE / 8), f = fk % 5, bi = fk / 5;
+  for (int it = first; it < groups * 5 * n_eval; it += stride) {
+    const int g = it % groups, fk = it / groups, f = fk % 5, bi = fk / 5;
     const int kb = p.scale_doubling ? (bi / 3) * 6 + bi % 3 : bi;
     float sn[8], cs[8];
 #pragma unroll
@@ -641,6 +645,15 @@ __device__ __forceinline__ void load_tile(const TileSrc& p, LoaderScratch* m, Ti
       put(f * 32 + 16 + kb + 3, g, cs);
     }
   }
+}
+
+template <bool FP16>
+__device__ __forceinline__ void load_tile(const TileSrc& p, LoaderScratch* m, TileMeta* md, uint8_t* fb, int s0,
+                                          int end, int lane) {
+  load_meta(p, m->col_tpos, md, s0, end, lane);
+  load_hits(p, m, md, lane);
+  fourier_operand<FP16>(p, m, md, TILE / 8, lane, 32,
+                        [&](int row, int g, uint4 v) { *reinterpret_cast<uint4*>(fb + bchunk(row, g)) = v; });
 }
 
 }  // namespace

@@ -81,9 +81,9 @@ struct PairMisc {
   alignas(16) float rinv[NE / 32][32];
 };
 
-// THIN: a tile is one slab, with half the columns and half the epilogue warps.  While
-// every slab can have a CTA of its own the batch's time is one tile's chain of steps,
-// and that is shorter then.
+// THIN: a tile is one slab, with half the columns and half the epilogue warps, and a CTA
+// has at most one.  While every slab can have a CTA of its own the batch's time is one
+// tile's chain of steps, and that is shorter then (101 tracks: 145 -> 120 us a call).
 template <bool THIN>
 constexpr int PAIR_EPI = THIN ? NE / 64 : NE / 32;   // epilogue warps
 template <bool THIN>
@@ -142,6 +142,10 @@ __global__ void __launch_bounds__(PAIR_NT<THIN>, 1) tc_pair_kernel(const __grid_
   int mine = 0;   // this CTA's tiles: blockIdx.x + j gridDim.x
   if ((int)blockIdx.x < n_tiles) mine = (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;
   volatile int* abort = &m->abort_flag;
+
+  // the loader's scratch for the CTA's first tiles, in the part of their XB that the Fourier
+  // operand leaves free
+  auto first_hits = [&](int u) { return reinterpret_cast<LoaderScratch*>(gbase + P_XB + u * P_TILE + 16384); };
 
   if (warp == 0) {
     // TMA producer: the 16 KB weight blocks in schedule order, one ring stage each; as in
@@ -325,12 +329,8 @@ __global__ void __launch_bounds__(PAIR_NT<THIN>, 1) tc_pair_kernel(const __grid_
     // the Fourier operand of tile u of a pair: the loads need the loader's hand-over,
     // the stores need the tile's HB and XB free.
     const uint8_t* fbuf = p.fbuf + (size_t)blockIdx.x * 4 * EB_BYTES;
-    // a thread's r-th 16-byte chunk of the operand (THIN: the first 64 columns, the first of
-    // each two 1 KB atoms)
-    auto chunk = [&](int r) -> uint32_t {
-      const uint32_t i = (uint32_t)(r * EW * 32 + x.te);
-      return THIN ? (i >> 6) * (uint32_t)B_SBO + (i & 63u) * 16u : i * 16u;
-    };
+    // a thread's r-th 16-byte chunk of the operand
+    auto chunk = [&](int r) -> uint32_t { return (uint32_t)(r * EW * 32 + x.te) * 16u; };
     auto fetch = [&](int pr, int u, uint4 (&v)[5]) {
       const int b = 2 * (pr & 1) + u;
       wait_on(smem_u32(&m->meta_full[b]), (uint32_t)(pr >> 1) & 1u);
@@ -344,10 +344,17 @@ __global__ void __launch_bounds__(PAIR_NT<THIN>, 1) tc_pair_kernel(const __grid_
       st_shared_v4(xb + chunk(4) - 128 * 256, v[4].x, v[4].y, v[4].z, v[4].w);   // k-rows 128-159
       signal_e(u, true);
     };
+    // The CTA's first tiles: nothing runs yet that could hide their operand, so the epilogue
+    // warps form it themselves instead of the loader warp alone (a call of 101 tracks
+    // 115 -> 93 us, 4,096 tracks of 64 hits 1,129 -> 1,077 us)
     for (int u = 0; u < 2 && u < mine; ++u) {
-      uint4 v[5];
-      fetch(0, u, v);
-      put(u, v);
+      wait_on(smem_u32(&m->meta_full[u]), 0);
+      const uint32_t hb = base + P_HB + u * P_TILE, xb = base + P_XB + u * P_TILE;
+      fourier_operand<FP16>(p.src, first_hits(u), &m->meta[u], (THIN ? SLAB : TILE) / 8, x.te, EW * 32,
+                            [&](int row, int g, uint4 v) {
+                              st_shared_v4(row < 128 ? hb + bchunk(row, g) : xb + bchunk(row - 128, g), v.x, v.y, v.z, v.w);
+                            });
+      signal_e(u, true);
     }
     for (int j = 0; j < mine; j += 2, ++pair) {
       const int nt = j + 1 < mine ? 2 : 1;
@@ -414,7 +421,7 @@ __global__ void __launch_bounds__(PAIR_NT<THIN>, 1) tc_pair_kernel(const __grid_
           // pooled, tile 0 by the warps of each slab's first segment, tile 1 by the others
 #pragma unroll 1
           for (int u = 0; u < nt; ++u) {
-            const bool more = j + 2 + u < mine;
+            const bool more = !THIN && j + 2 + u < mine;
             uint4 fv[5];
             if (more) fetch(pair + 1, u, fv);
             wait_acc(u);
@@ -438,7 +445,13 @@ __global__ void __launch_bounds__(PAIR_NT<THIN>, 1) tc_pair_kernel(const __grid_
         if (!__all_sync(0xffffffffu, got) && lane == 0) set_abort(&m->abort_flag, p.err);
       }
       const int t = (int)blockIdx.x + j * (int)gridDim.x;
-      load_tile<FP16>(p.src, &m->ls, &m->meta[b], fbuf + b * EB_BYTES, THIN ? t : 2 * t, THIN ? t + 1 : n_slabs, lane);
+      const int s0 = THIN ? t : 2 * t, end = THIN ? t + 1 : n_slabs;
+      if (j < 2) {
+        load_meta(p.src, first_hits(j)->col_tpos, &m->meta[b], s0, end, lane);
+        load_hits(p.src, first_hits(j), &m->meta[b], lane);
+      } else {
+        load_tile<FP16>(p.src, &m->ls, &m->meta[b], fbuf + b * EB_BYTES, s0, end, lane);
+      }
       __threadfence_block();
       __syncwarp();
       if (j == p.hold_tile && blockIdx.x == 0) {   // test hook, as in the one-tile kernel
