@@ -408,14 +408,22 @@ extern "C" int trackfit_forward_host(trackfit_t h, const float* hits_host, const
   }
   cudaStream_t cs = h->cp_stream;
   cudaEvent_t* ev = h->cp_ev;
-  const int64_t chunk = TF_HOST_CHUNK;
-  const int64_t n_chunks = (n_tracks + chunk - 1) / chunk;
+  // Only the first step's copy is not hidden, so that step is short: its copy takes 0.08 ms
+  // instead of 0.6 ms at 24 hits a track (300,001 tracks of d_model 256: see the header for
+  // the steps).
+  const int64_t chunk = TF_HOST_CHUNK, head = n_tracks < TF_HOST_FIRST ? n_tracks : TF_HOST_FIRST;
+  const int64_t n_chunks = 1 + (n_tracks - head + chunk - 1) / chunk;
+  auto start = [&](int64_t k) { return k == 0 ? 0 : head + (k - 1) * chunk; };
+  auto count = [&](int64_t k) {
+    const int64_t most = k == 0 ? head : chunk;
+    return n_tracks - start(k) < most ? n_tracks - start(k) : most;
+  };
   // chunk k's events: in(k) (its inputs have landed), done(k) (its outputs are
   // computed), from a ring (each is waited for before it is recorded again)
   auto ev_in = [&](int64_t k) { return ev[1 + (2 * k) % (TF_HOST_EVENTS - 2)]; };
   auto ev_done = [&](int64_t k) { return ev[2 + (2 * k) % (TF_HOST_EVENTS - 2)]; };
   auto send = [&](int64_t k) -> cudaError_t {   // chunk k's inputs, on the copy stream
-    const int64_t c0 = k * chunk, nb = (n_tracks - c0 < chunk) ? n_tracks - c0 : chunk;
+    const int64_t c0 = start(k), nb = count(k);
     cudaError_t r = cudaMemcpyAsync(h->st_hits + c0 * row, hits_host + c0 * row, nb * row * sizeof(float),
                                     cudaMemcpyHostToDevice, cs);
     if (r == cudaSuccess)
@@ -433,7 +441,7 @@ extern "C" int trackfit_forward_host(trackfit_t h, const float* hits_host, const
     if (k + 1 < n_chunks) e = send(k + 1);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ev_in(k), 0);
     if (e != cudaSuccess) break;
-    const int64_t c0 = k * chunk, nb = (n_tracks - c0 < chunk) ? n_tracks - c0 : chunk;
+    const int64_t c0 = start(k), nb = count(k);
     const int r = trackfit_forward(h, h->st_hits + c0 * row, h->st_n + c0, nb, h->st_out + c0 * 5, stream);
     if (r != TRACKFIT_OK) {
       cudaStreamSynchronize(cs);
