@@ -363,7 +363,7 @@ extern "C" int trackfit_forward_host(trackfit_t h, const float* hits_host, const
   tf_nvtx_range nvtx_range("trackfit_forward_host");
   if (!h || !hits_host || !n_hits_host || !out_host || n_tracks <= 0) return TRACKFIT_ERR_INVALID_ARG;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  const size_t row = (size_t)h->s.T * 5;
+  const size_t row = (size_t)h->s.T * h->s.F;
   if (n_tracks > h->st_cap) {
     cudaStreamSynchronize(st);
     tf_free(h->st_hits);

@@ -327,7 +327,7 @@ int tf_simt_run(const tf_shape& s, const tf_blob_off& o, const float* W, float* 
     float* PR = XH + R * D;
     float* Y = PR + R * PD;
     float* X1 = Y + R * YW;
-    const float* hc = offs ? hits : hits + c0 * s.T * 5;
+    const float* hc = offs ? hits : hits + c0 * s.T * s.F;
     const int64_t* oc = offs ? offs + c0 : nullptr;
     const int32_t* nc = n_hits + c0;
     if (prof) tf_prof_begin(prof, st);

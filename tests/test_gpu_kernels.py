@@ -205,3 +205,20 @@ def test_packing_segments_do_not_matter_to_a_track(T, n, hits):
     got, (_, n_bad) = forward(T, m, blob, h[:n], nh[:n])
     assert n_bad == 1
     np.testing.assert_array_equal(got, want[:n])
+
+
+def test_hit_rows_of_fifteen_features_in_host_buffers_and_chunks(T):
+    """Hit rows wider than five features: from host buffers (copied whole, in two steps),
+    and on the CUDA cores past the workspace's first chunk of tracks (4,923 of these)."""
+    w = W.workload("paper", n_tracks=33000)
+    tb = W.gen_tracks(w)
+    hits, blob = W.paper_hits(tb, w), W.gen_weights(w.model, 2)
+    want, _ = forward(T, w.model, blob, hits, tb.n_hits)
+    out = np.full((33000, 5), -7.0, np.float32)
+    with T.Trackfit(w.model, blob) as tf:
+        tf.forward_host(hits, tb.n_hits, out)
+    np.testing.assert_array_equal(out, want)
+    m = w.model.with_(precision=W.PRECISION_FP32)
+    got, _ = forward(T, m, blob, hits[:5200], tb.n_hits[:5200])
+    few, _ = forward(T, m, blob, hits[5000:5200], tb.n_hits[5000:5200])
+    np.testing.assert_array_equal(got[5000:], few)
