@@ -40,7 +40,8 @@ from paper_2609_32479_gb300 import workloads as W  # noqa: E402
 
 METRIC = "tracks/sec at 1 GB300 (device-timed) and % of HBM/tensor roofline vs CPU oracle"
 FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}
-KERNEL_SRC = os.path.join(ROOT, "paper_2609_32479_gb300", "csrc", "tc_forward.cu")
+KERNEL_SRC = tuple(os.path.join(ROOT, "paper_2609_32479_gb300", "csrc", f)
+                   for f in ("tc_forward.cu", "tc_epilogue.cuh"))
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "tc_forward_large.traffic.json")
 
 
@@ -440,28 +441,6 @@ def product_flops(m, n_hits):
     return int(np.asarray(n_hits, dtype=np.int64).sum()) * per_hit
 
 
-def product_bytes(m, n_hits):
-    """Algorithmic HBM bytes of the per-hit products over the valid hits: each
-    product reads its 16-bit operand rows (and, with a residual, the fp32 stream)
-    and writes its results (fp32 projections and residual stream, 16-bit operands
-    of the next product); the weights stay in L2."""
-    D, H, E = m.d_model, m.d_hidden, m.embed_dim
-    per_hit = 2 * E + 2 * D                       # e1: Fourier operand in, SiLU operand out
-    if m.topology == W.TOPOLOGY_ATTENTION:
-        per_hit += 2 * D + 4 * D + 2 * D          # e2: x and its pre-norm operand
-        for l in range(m.n_layers):
-            last = l + 1 == m.n_layers
-            per_hit += 2 * D + 4 * 3 * D          # q, k, v
-            per_hit += 2 * D + 4 * D + 4 * D + 2 * D   # W_o: operand, residual in, x' and its pre-norm out
-            per_hit += 2 * D + 2 * H              # W_1: SiLU operand out
-            per_hit += 2 * H + 4 * D + 4 * D + (0 if last else 2 * D)   # W_2
-    else:
-        per_hit += 2 * D + 2 * D                  # e2: the first layer's operand
-        for l in range(m.n_layers):
-            per_hit += 2 * (D if l == 0 else 2 * H) + 4 * 4 * H
-    return int(np.asarray(n_hits, dtype=np.int64).sum()) * per_hit
-
-
 PAPER_CONTEXT = {"paper": "the paper reports 5.41 M tracks/s on one H100 NVL for its trained minGRU model on its data",
                  "transformer": "the paper reports 3.18 M tracks/s on one H100 NVL for its Transformer of the same "
                                 "parameter count (Tab. A.1)"}
@@ -500,7 +479,7 @@ def paper_main(args, name="paper"):
             step()
         ms = _time_events(step, reps, stream)
         enc_ms = _time_events(lambda: tf.forward(hits, nh, corr, stream), reps, stream)
-        # the product kernel's own launches, timed by the library's hook in a
+        # the encoder kernel's own launches, timed by the library's hook in a
         # separate pass (the hook synchronises between batches of launches)
         tf.profile(True)
         tf.profile_read()
@@ -512,16 +491,14 @@ def paper_main(args, name="paper"):
         path = tf.path
     D, H = m.d_model, m.d_hidden
     if path.startswith("tcgen05-rows"):
-        # the products are contractions of K = 128-480 with fp32 results: far below
-        # the tensor pipe's ridge point, so HBM bounds them
+        # one kernel holds every product of a tile, with its activations on the SM
         peaks, peak_kind = load_peaks()
-        peak = float(peaks.get("hbm_gbs", FALLBACK_PEAKS["hbm_gbs"]))
-        ach = reps * product_bytes(m, tb.n_hits) / (kern_ms * 1e-3) / 1e9
-        tfl = reps * product_flops(m, tb.n_hits) / (kern_ms * 1e-3) / 1e12
-        roof = {"bound": "hbm", "kernel": "row_gemm_kernel (tcgen05 fp16 products over valid hit rows)",
-                "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak, "traffic": None,
-                "peak_kind": f"{peak_kind} copy bandwidth",
-                "bytes_per_valid_hit": product_bytes(m, [1]), "tensor_tflops": tfl,
+        peak = float(peaks.get("bf16_tflops", FALLBACK_PEAKS["bf16_tflops"]))
+        ach = reps * product_flops(m, tb.n_hits) / (kern_ms * 1e-3) / 1e12
+        kern = "concat_kernel" if m.topology == W.TOPOLOGY_CONCAT else "transformer_kernel"
+        roof = {"bound": "tensor", "kernel": f"{kern} (tcgen05 fp16, whole encoder)",
+                "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak, "traffic": None,
+                "peak_kind": f"{peak_kind} cuBLAS bf16 burst (fp16 runs at the same rate)",
                 "launches_per_step": kern_n // reps, "kernel_ms_per_step": kern_ms / reps}
     else:
         ach = encoder_flops(m, tb.n_hits) / (enc_ms * 1e-3) / 1e12
@@ -546,13 +523,15 @@ def paper_main(args, name="paper"):
     return 0
 
 
-def code_digest(path: str) -> str:
-    """sha256 of a CUDA source's code: comments removed and whitespace collapsed, so
+def code_digest(paths) -> str:
+    """sha256 of CUDA sources' code: comments removed and whitespace collapsed, so
     that an edit of the comments alone keeps the digest (the compiled kernel is the
     same) and any change of the code changes it."""
     import re
-    with open(path) as fh:
-        src = fh.read()
+    src = ""
+    for path in paths:
+        with open(path) as fh:
+            src += fh.read() + "\n"
     src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)
     src = re.sub(r"//[^\n]*", " ", src)
     return hashlib.sha256(" ".join(src.split()).encode()).hexdigest()
@@ -722,7 +701,8 @@ def main():
                 "frac": (achieved / peak) if achieved else None, "traffic": traffic,
                 "peak_kind": peak_kind,
                 "frac_of_sustained": (achieved / peak_sus) if achieved else None,
-                "kernel": "tc_forward_kernel" if tf.path.startswith("tcgen05") else "simt layer sequence",
+                "kernel": ("tc_pair_kernel" if m.d_model == 128 else "tc_forward_kernel") if tf.path.startswith("tcgen05")
+                          else "encoder_fp32_kernel",
                 "kernel_ms_avg": kern_avg_s * 1e3, "launches_per_step": launches_per_step,
                 "flops_per_launch": flops_launch,
                 "algorithmic_bytes_per_launch": B * bytes_per_track(m) / launches_per_step,
@@ -736,8 +716,8 @@ def main():
             "path": tf.path, "roofline": roofline, "clocks": clk,
             "e2e": {"value": e2e_value, "unit": "tracks/s", "h2d_bytes_per_step": int(tb.hits.nbytes + tb.n_hits.nbytes),
                     "d2h_bytes_per_step": int(B * 5 * 4), "matches_device_result": same},
-            # per launch chunk: three packing kernels, the fused encoder, the head
-            "gpu_launches": int(5 * math.ceil(B / 1048576) * args.steps) if tf.path.startswith("tcgen05") else None,
+            # per launch chunk: the packing, the fused encoder, the head
+            "gpu_launches": int(3 * math.ceil(B / 1048576) * args.steps) if tf.path.startswith("tcgen05") else None,
             "device_errors": {"status": st, "bad_tracks": nbad}}
     if not args.no_cpu_baseline and world == 1:
         pool = OraclePool(w)
