@@ -3,7 +3,9 @@
 // features against that helix (asinh du, asinh dv in the curvilinear frame,
 // path length s); plus the decode of the heads' corrections against the seed
 // (Sec. 3.3).  A thread fits a track's seed, then the threads of a CTA share the
-// hits of its tracks.
+// hits of its tracks.  Bound by the fp64 pipe (524,288 tracks with the features:
+// 7.20 ms with a thread for all of a track's hits and a sine and cosine a Newton
+// step, 2.65 ms with rotations and starts from fp32).
 //
 // Conventions (those of the synthetic track generator): B along +z; a positive
 // charge turns clockwise seen from +z; at turning angle a from the perigee the
