@@ -87,9 +87,11 @@ typedef enum {
  * constants (feat_max > feat_min); fourier_scale[k] = s_k, the feature argument is
  * pi * s_k * u; rms_eps > 0.  The fused tensor-core path runs 16-bit-operand
  * MERGE configs with 5 features, mean pooling and d_model 128 or 256; the
- * packed-row tensor-core path runs 16-bit-operand CONCAT and ATTENTION configs
- * (valid hits only, one tensor-core product per matrix of Sec. 3.2 / App. A.3);
- * everything else runs on the CUDA cores. */
+ * tensor-core rows path runs 16-bit-operand CONCAT and ATTENTION configs (valid hits
+ * only), the paper's sizes in one kernel for the whole encoder, other sizes with one
+ * tensor-core product per matrix of Sec. 3.2 / App. A.3; everything else runs on the
+ * CUDA cores, fp32 MERGE configs of d_model up to 128 (as far as shared memory
+ * holds their rows) in one fused kernel. */
 typedef struct {
   int32_t abi_version;
   int32_t max_hits;
@@ -194,8 +196,8 @@ int trackfit_forward_packed(trackfit_t h, const float* hits, int64_t n_hit_rows,
  * End-to-end variant with HOST buffers: copies hits [n_tracks][max_hits][5] and
  * n_hits [n_tracks] to the device, runs the encoder and copies out_params
  * [n_tracks][5] back, all on `stream`, and returns after the stream has finished
- * this work (synchronous).  The batch moves in steps of 262,144 tracks, the first of 32,768: a
- * step's inputs are copied on a stream of the handle's own while the previous
+ * this work (synchronous).  The batch moves in steps of 262,144 tracks, the
+ * first of 32,768: a step's inputs are copied on a stream of the handle's own while the previous
  * step computes on `stream` (only the first step's copy is not hidden), and
  * its outputs are copied back behind it.  Pinned
  * (page-locked) host memory makes the copies asynchronous and lets them
@@ -231,8 +233,8 @@ const char* trackfit_path_name(trackfit_t h);
 int trackfit_set_path(trackfit_t h, int path);
 
 /* Timing hook: with enable = 1 every forward records CUDA events on its stream
- * around the main compute kernel (the fused tcgen05 kernel, every product
- * launch of the packed-row tcgen05 path, or the SIMT layer sequence);
+ * around the main compute kernel (the fused encoder kernel, every product launch
+ * of the layer-by-layer rows path, or the SIMT layer sequence);
  * trackfit_profile_read synchronises on them, returns the summed
  * kernel time in milliseconds and the number of timed launches since the last
  * read, and resets both.  enable = 0 releases the events. */
