@@ -334,8 +334,8 @@ int trackfit_seed(const float* hits, int32_t hit_stride, const int32_t* n_hits, 
 int trackfit_decode(const double* seed, const float* corrections, int64_t n_tracks, float* out_params,
                     void* stream);
 
-/* Test hook for the failure path of the fused tensor-core kernel's bounded
- * waits (every wait for a hand-over inside that kernel gives up after a time
+/* Test hook for the failure path of the fused tensor-core kernels' bounded
+ * waits (every wait for a hand-over inside such a kernel gives up after a time
  * limit, records TRACKFIT_ERR_TIMEOUT in the handle's device error counters,
  * and the kernel drains its copies and products and returns instead of
  * hanging).  For this handle's later forwards: limit_ns > 0 replaces the 2 s
@@ -345,11 +345,12 @@ int trackfit_decode(const double* seed, const float* corrections, int64_t n_trac
  * expires; -1 holds nothing.  The outputs of a forward that timed out are not
  * valid; trackfit_device_errors reports TRACKFIT_ERR_TIMEOUT and resets the
  * counters, after which the handle is usable again.  Host side only; launches
- * nothing.  On a handle of the packed-row tensor-core path (16-bit CONCAT and
- * ATTENTION configs) only the limit applies: hold_tile must be -1 there.
+ * nothing.  On a handle of the tensor-core rows path that runs one product per
+ * matrix (16-bit CONCAT and ATTENTION configs that no fused kernel takes) only the
+ * limit applies: hold_tile must be -1 there.
  * Errors: INVALID_ARG (NULL handle, limit_ns < 0, hold_tile < -1), UNSUPPORTED
  * (the handle runs the CUDA-core path, which has no waits, or hold_tile >= 0 on
- * the packed-row path). */
+ * a rows handle without a fused kernel). */
 int trackfit_debug_wait_limit(trackfit_t h, int64_t limit_ns, int32_t hold_tile);
 
 /* Test hook for allocation failures (host side, not thread-safe): every device

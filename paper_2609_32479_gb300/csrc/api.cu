@@ -53,11 +53,7 @@ extern "C" int64_t trackfit_debug_alloc(int64_t fail_nth, int64_t* attempted) {
 
 extern "C" int trackfit_debug_wait_limit(trackfit_t h, int64_t limit_ns, int32_t hold_tile) {
   if (!h) return TRACKFIT_ERR_INVALID_ARG;
-  if (h->rows) {   // the packed-row path: the limit only (it has no loader hand-over to hold)
-    if (limit_ns < 0 || hold_tile != -1) return limit_ns < 0 || hold_tile < -1 ? TRACKFIT_ERR_INVALID_ARG
-                                                                               : TRACKFIT_ERR_UNSUPPORTED;
-    return tf_rows_wait_limit(h, limit_ns);
-  }
+  if (h->rows) return tf_rows_wait_limit(h, limit_ns, hold_tile);
   return tf_tc_wait_limit(h, limit_ns, hold_tile);
 }
 

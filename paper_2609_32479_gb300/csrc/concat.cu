@@ -45,6 +45,7 @@ struct CatParams {
   const float* b_in;            // [L][NDC * 256], chunk order
   unsigned long long* err;
   uint64_t wait_ns;
+  int hold_tile;        // test hook: CTA 0's loader holds this tile's metadata hand-over (-1: none)
 };
 
 struct CatMisc {
@@ -248,7 +249,10 @@ __global__ void __launch_bounds__(NT, 1) concat_kernel(const __grid_constant__ C
     // (16 arrivals).  One operand barrier is enough: between two operand hand-overs every
     // warp waits for a product that the issuer starts only after the first of them.  A
     // failed wait sets the abort flag and every later wait fails fast, but no warp leaves
-    // the loop early (the segments of a slab meet at named barriers).
+    // the loop early (the segments of a slab meet at named barriers).  `alive` (the same for
+    // a warp's lanes): every wait of this warp has succeeded; only then is the metadata of its
+    // tile complete and kept until the warp releases it, and may an address be formed from it.
+    bool alive = true;
     ECtx x;
     x.q = warp & 3;
     x.seg = (warp - 2) >> 2;
@@ -259,12 +263,14 @@ __global__ void __launch_bounds__(NT, 1) concat_kernel(const __grid_constant__ C
     x.col0 = SEGW * x.seg;
     x.te = threadIdx.x - 64;
     x.pool = p.pool;
-    x.abort_flag = &m->abort_flag;
     const uint32_t tq = tmem + ((uint32_t)(32 * x.q) << 16);
     uint32_t g = 0;
     auto wait_on = [&](uint32_t bar, uint32_t parity) {
       const bool got = mbar_wait(bar, parity, abort, p.wait_ns);
-      if (!__all_sync(0xffffffffu, got) && lane == 0) cat_abort(m, p.err);
+      if (!__all_sync(0xffffffffu, got)) {
+        if (lane == 0) cat_abort(m, p.err);
+        alive = false;
+      }
       tc_fence_after();
     };
     auto arrive = [&](uint32_t bar, bool wrote_operands) {
@@ -314,7 +320,7 @@ __global__ void __launch_bounds__(NT, 1) concat_kernel(const __grid_constant__ C
           scan_chain<true>(x, z, n);
           if (!last) {
             store_row32<FP16>(base + CT_Y + dc * 32768, x.c, x.col0, z);
-          } else if (!*abort) {   // after an expired wait the metadata may be missing
+          } else if (alive) {
             put_endpoints(x, z, (x.c >> 6) * CT_H + dc * 64 + (x.c & 63));
           }
         }
@@ -330,9 +336,14 @@ __global__ void __launch_bounds__(NT, 1) concat_kernel(const __grid_constant__ C
       if (i >= 2) {
         const bool got = mbar_wait(smem_u32(&m->meta_free[b]), (uint32_t)((i >> 1) - 1) & 1u, abort, p.wait_ns);
         if (!__all_sync(0xffffffffu, got) && lane == 0) cat_abort(m, p.err);
+        // after a failure anywhere a release may have come from a warp that gave up: stop, so
+        // that the metadata others still read stays as it is
+        if (!__all_sync(0xffffffffu, got && !*abort)) break;
       }
       load_meta(p.src, nullptr, &m->meta[b], 2 * t, n_slabs, lane);
       __threadfence_block();
+      __syncwarp();
+      if (i == p.hold_tile && blockIdx.x == 0) hold_hand_over(abort, p.wait_ns);
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&m->meta_full[b]));
     }
@@ -456,13 +467,14 @@ int tf_cat_create(trackfit_ctx* h, const float* W, tf_cat_state** out) {
   return TRACKFIT_OK;
 }
 
-int tf_cat_forward(trackfit_ctx* h, tf_cat_state* c, uint64_t wait_ns, const float* hits, const int32_t* n_hits,
-                   int64_t B, float* out, float* out_q, float* out_pool, cudaStream_t st, const int64_t* offs) {
+int tf_cat_forward(trackfit_ctx* h, tf_cat_state* c, uint64_t wait_ns, int hold_tile, const float* hits,
+                   const int32_t* n_hits, int64_t B, float* out, float* out_q, float* out_pool, cudaStream_t st, const int64_t* offs) {
   const tf_shape& s = h->s;
   CatParams p = c->p;
   const bool fp16 = s.precision == TRACKFIT_FP16_PROJ;
   p.err = h->d_err;
   p.wait_ns = wait_ns;
+  p.hold_tile = hold_tile;
   p.src.T = s.T;
   const tf_pack pk = tf_pack_in(c->pack, c->chunk);
   p.src.slab = pk.slab;

@@ -616,7 +616,7 @@ __global__ void pool_mean_rows_kernel(const float* __restrict__ x, const int64_t
 // ------------------------------------------------------------------ host side
 struct tf_rows_state {
   // the configurations that concat.cu or transformer.cu takes: nothing below but
-  // wait_ns is set up then
+  // wait_ns and hold_tile is set up then
   tf_cat_state* cat;
   tf_tr_state* tr;
   int fp16;
@@ -633,6 +633,7 @@ struct tf_rows_state {
   RowGemm lay[TF_MAX_LAYERS][4];
   size_t smem;
   uint64_t wait_ns;
+  int hold_tile;            // test hook, for cat and tr
 };
 
 namespace {
@@ -785,9 +786,13 @@ void tf_rows_destroy(trackfit_ctx* h) {
   h->rows = nullptr;
 }
 
-int tf_rows_wait_limit(trackfit_ctx* h, int64_t limit_ns) {
-  if (!h->rows) return TRACKFIT_ERR_UNSUPPORTED;
-  h->rows->wait_ns = limit_ns > 0 ? (uint64_t)limit_ns : RG_WAIT_NS;
+int tf_rows_wait_limit(trackfit_ctx* h, int64_t limit_ns, int hold_tile) {
+  tf_rows_state* r = h->rows;
+  if (!r) return TRACKFIT_ERR_UNSUPPORTED;
+  if (limit_ns < 0 || hold_tile < -1) return TRACKFIT_ERR_INVALID_ARG;
+  if (hold_tile != -1 && !r->cat && !r->tr) return TRACKFIT_ERR_UNSUPPORTED;   // the products have no loader to hold
+  r->wait_ns = limit_ns > 0 ? (uint64_t)limit_ns : RG_WAIT_NS;
+  r->hold_tile = hold_tile;
   return TRACKFIT_OK;
 }
 
@@ -799,6 +804,7 @@ int tf_rows_create(trackfit_ctx* h, const float* host_w) {
   h->rows = r;   // freed by tf_rows_destroy on any failure below
   r->fp16 = s.precision == TRACKFIT_FP16_PROJ;
   r->wait_ns = RG_WAIT_NS;
+  r->hold_tile = -1;
   if (tf_cat_supported(s)) return tf_cat_create(h, host_w, &r->cat);
   if (tf_tr_supported(s)) return tf_tr_create(h, host_w, &r->tr);
   r->doubling = 1;
@@ -1031,8 +1037,8 @@ int tf_rows_forward(trackfit_ctx* h, const float* hits, const int32_t* n_hits, i
                     float* out_q, float* out_pool, cudaStream_t st, const int64_t* offs) {
   tf_rows_state* r = h->rows;
   const tf_shape& s = h->s;
-  if (r->cat) return tf_cat_forward(h, r->cat, r->wait_ns, hits, n_hits, B, out, out_q, out_pool, st, offs);
-  if (r->tr) return tf_tr_forward(h, r->tr, r->wait_ns, hits, n_hits, B, out, out_q, out_pool, st, offs);
+  if (r->cat) return tf_cat_forward(h, r->cat, r->wait_ns, r->hold_tile, hits, n_hits, B, out, out_q, out_pool, st, offs);
+  if (r->tr) return tf_tr_forward(h, r->tr, r->wait_ns, r->hold_tile, hits, n_hits, B, out, out_q, out_pool, st, offs);
   for (int64_t c0 = 0; c0 < B; c0 += r->chunk) {
     const int64_t nb = B - c0 < r->chunk ? B - c0 : r->chunk;
     const float* hc = offs ? hits : hits + c0 * s.T * s.F;

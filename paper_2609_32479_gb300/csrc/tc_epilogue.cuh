@@ -174,7 +174,6 @@ struct ECtx {
   float (*part)[TILE];  // partial column sums of the four quadrants
   float (*carry)[128];  // [slab][channel]: scan states between a slab's column segments
   float* rinv;          // the warp's 32 inverse RMS values
-  int* abort_flag;
   float* pool;
   float rms_eps;
   // quadrant q (TMEM lanes / channels 32q..), column segment seg = 32-column
@@ -363,16 +362,14 @@ __device__ __forceinline__ void ep_residual(const ECtx& x, const float* bias, co
   }
 }
 
-// Masked mean pooling of the last layer's output X = acc + bias.  The warp of
+// Masked mean pooling of the last layer's output X = acc + bias, only with the tile's
+// metadata at hand (its stores are indexed by it).  The warp of
 // quadrant q and slab half pools channel tile mt (channels 128 mt + 32 q + lane)
 // over all 64 columns of the slab, each track's hits summed in order from its
 // first: the two warps of a slab's segments take different channel tiles, or
 // different hit tiles.  The column loops stay rolled: this runs once per tile, and its code is cold.
 template <int MT>
 __device__ __forceinline__ void ep_pool(const ECtx& x, int mt, const float* bias) {
-  // after an expired wait the tile's metadata may not have been handed over:
-  // no stores indexed by it
-  if (*reinterpret_cast<volatile int*>(x.abort_flag)) return;
   constexpr int D = 128 * MT;
   const int ch = mt * 128 + x.c;
   const float bv = bias[ch];
@@ -514,6 +511,15 @@ template <bool FP16>
 __device__ __forceinline__ void scan_chain_store(const ECtx& x, float (&a)[32], const float (&b)[32]) {
   scan_chain<false>(x, a, b);
   store_row32<FP16>(x.hb, x.c, x.col0, a);
+}
+
+// Test hook: hold a loader's hand-over past the waiters' limit (at most twice the limit, and
+// no longer once a wait has given up), so that the epilogue's wait for it expires; the
+// metadata itself is complete.
+__device__ __forceinline__ void hold_hand_over(volatile int* abort, uint64_t wait_ns) {
+  const uint64_t t0 = globaltimer();
+  while (!*abort && globaltimer() - t0 < 2 * wait_ns) {
+  }
 }
 
 // Tile set-up, run one tile ahead by the loader warp while the epilogue warps

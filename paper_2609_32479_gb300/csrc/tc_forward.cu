@@ -382,7 +382,6 @@ __global__ void __launch_bounds__(NT, 1) tc_forward_kernel(const __grid_constant
     x.part = m->part;
     x.carry = m->carry;
     x.rinv = m->rinv[warp - 2];
-    x.abort_flag = &m->abort_flag;
     x.pool = p.pool;
     x.rms_eps = p.rms_eps;
     uint32_t acc_ph0 = 0, acc_ph1 = 0, hb_phase = 0;
@@ -405,7 +404,11 @@ __global__ void __launch_bounds__(NT, 1) tc_forward_kernel(const __grid_constant
     // A failed wait sets the abort flag and every later wait fails fast, but no
     // warp leaves the loop early: all warps keep taking the same sequence of named
     // barriers (the column-norm exchanges, the segment hand-overs), so none of
-    // them can be left waiting.
+    // them can be left waiting.  `alive` (the same for a warp's lanes): every wait of
+    // this warp has succeeded.  Only then is the metadata of its tile complete and kept
+    // until the warp releases it (the loader stops at the first failure), so only then may
+    // an address be formed from it.
+    bool alive = true;
     auto signal_to = [&](uint32_t bar, bool wrote_operands) {
       if (wrote_operands) fence_proxy_async_smem();   // costly: only after operand writes
       tc_fence_before();
@@ -420,7 +423,10 @@ __global__ void __launch_bounds__(NT, 1) tc_forward_kernel(const __grid_constant
     auto signal = [&]() { signal_e(true); };
     auto wait_on = [&](uint32_t bar, uint32_t& ph) {
       const bool got = mbar_wait(bar, ph, abort, p.wait_ns);   // try_wait: suspends instead of polling
-      if (!__all_sync(0xffffffffu, got) && x.lane == 0) set_abort(&m->abort_flag, p.err);
+      if (!__all_sync(0xffffffffu, got)) {
+        if (x.lane == 0) set_abort(&m->abort_flag, p.err);
+        alive = false;
+      }
       ph ^= 1u;
       tc_fence_after();
     };
@@ -514,7 +520,7 @@ __global__ void __launch_bounds__(NT, 1) tc_forward_kernel(const __grid_constant
           wait_acc();
           wait_acc();
           if (more) tile_put(fv);
-          ep_pool<2>(x, x.sub, p.b_2 + (size_t)l * p.D);
+          if (alive) ep_pool<2>(x, x.sub, p.b_2 + (size_t)l * p.D);
           signal_to(smem_u32(&m->meta_free[i & 1]), false);   // this tile's metadata is no longer read
         }
       }
@@ -529,6 +535,9 @@ __global__ void __launch_bounds__(NT, 1) tc_forward_kernel(const __grid_constant
       if (i >= 2) {   // buffer b last held the metadata of tile i - 2
         const bool got = mbar_wait(smem_u32(&m->meta_free[b]), free_ph[b], abort, p.wait_ns);
         if (!__all_sync(0xffffffffu, got) && lane == 0) set_abort(&m->abort_flag, p.err);
+        // after a failure anywhere a release may have come from a warp that gave up: stop, so
+        // that the metadata others still read stays as it is
+        if (!__all_sync(0xffffffffu, got && !*abort)) break;
         free_ph[b] ^= 1u;
       }
       if (i == 0) {
@@ -539,14 +548,7 @@ __global__ void __launch_bounds__(NT, 1) tc_forward_kernel(const __grid_constant
       }
       __threadfence_block();
       __syncwarp();
-      if (i == p.hold_tile && blockIdx.x == 0) {
-        // test hook: hold this hand-over past the waiters' limit (at most twice
-        // the limit, and no longer once a wait has given up), so that the
-        // epilogue's wait for it expires; the metadata itself is complete
-        const uint64_t t0 = globaltimer();
-        while (!*abort && globaltimer() - t0 < 2 * p.wait_ns) {
-        }
-      }
+      if (i == p.hold_tile && blockIdx.x == 0) hold_hand_over(abort, p.wait_ns);
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&m->meta_full[b]));
     }

@@ -272,7 +272,9 @@ __global__ void __launch_bounds__(PAIR_NT<THIN>, 1) tc_pair_kernel(const __grid_
     // Epilogue: every step for tile 0, then for tile 1.  The warps run decoupled, as in
     // the one-tile kernel; its argument that no warp is two hand-overs ahead or two
     // commits behind holds for each tile's own barriers.  A failed wait sets the abort
-    // flag and every later wait fails fast, but no warp leaves the loop early.
+    // flag and every later wait fails fast, but no warp leaves the loop early; `alive` as in
+    // the one-tile kernel.
+    bool alive = true;
     const int q = warp & 3, seg = (warp - 2) >> 2;
     ECtx x;
     x.q = q;
@@ -285,7 +287,6 @@ __global__ void __launch_bounds__(PAIR_NT<THIN>, 1) tc_pair_kernel(const __grid_
     x.te = threadIdx.x - 64;
     x.zn = tmem + ((uint32_t)(32 * q) << 16) + 256;
     x.rinv = m->rinv[warp - 2];
-    x.abort_flag = &m->abort_flag;
     x.pool = p.pool;
     x.rms_eps = p.rms_eps;
     int pair = 0;
@@ -313,7 +314,10 @@ __global__ void __launch_bounds__(PAIR_NT<THIN>, 1) tc_pair_kernel(const __grid_
     };
     auto wait_on = [&](uint32_t bar, uint32_t parity) {
       const bool got = mbar_wait(bar, parity, abort, p.wait_ns);
-      if (!__all_sync(0xffffffffu, got) && lane == 0) set_abort(&m->abort_flag, p.err);
+      if (!__all_sync(0xffffffffu, got)) {
+        if (lane == 0) set_abort(&m->abort_flag, p.err);
+        alive = false;
+      }
       tc_fence_after();
     };
     auto wait_acc = [&](int u) {
@@ -427,7 +431,7 @@ __global__ void __launch_bounds__(PAIR_NT<THIN>, 1) tc_pair_kernel(const __grid_
             wait_acc(u);
             if (more) put(u, fv);
           }
-          if (x.sub < nt) {
+          if (alive && x.sub < nt) {
             tile(x.sub);
             ep_pool<1>(x, 0, p.b_2 + (size_t)l * 128);
           }
@@ -443,6 +447,7 @@ __global__ void __launch_bounds__(PAIR_NT<THIN>, 1) tc_pair_kernel(const __grid_
       if (pr >= 2) {   // the buffer last held a tile of pair pr - 2
         const bool got = mbar_wait(smem_u32(&m->meta_free[b]), (uint32_t)((pr >> 1) - 1) & 1u, abort, p.wait_ns);
         if (!__all_sync(0xffffffffu, got) && lane == 0) set_abort(&m->abort_flag, p.err);
+        if (!__all_sync(0xffffffffu, got && !*abort)) break;   // as in the one-tile kernel
       }
       const int t = (int)blockIdx.x + j * (int)gridDim.x;
       const int s0 = THIN ? t : 2 * t, end = THIN ? t + 1 : n_slabs;
@@ -454,11 +459,7 @@ __global__ void __launch_bounds__(PAIR_NT<THIN>, 1) tc_pair_kernel(const __grid_
       }
       __threadfence_block();
       __syncwarp();
-      if (j == p.hold_tile && blockIdx.x == 0) {   // test hook, as in the one-tile kernel
-        const uint64_t t0 = globaltimer();
-        while (!*abort && globaltimer() - t0 < 2 * p.wait_ns) {
-        }
-      }
+      if (j == p.hold_tile && blockIdx.x == 0) hold_hand_over(abort, p.wait_ns);
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&m->meta_full[b]));
     }

@@ -170,16 +170,16 @@ struct tf_cat_state;
 bool tf_cat_supported(const tf_shape& s);
 int tf_cat_create(trackfit_ctx* h, const float* host_w, tf_cat_state** out);
 void tf_cat_destroy(tf_cat_state* c);
-int tf_cat_forward(trackfit_ctx* h, tf_cat_state* c, uint64_t wait_ns, const float* hits, const int32_t* n_hits,
-                   int64_t B, float* out, float* out_q, float* out_pool, cudaStream_t st, const int64_t* offs);
+int tf_cat_forward(trackfit_ctx* h, tf_cat_state* c, uint64_t wait_ns, int hold_tile, const float* hits,
+                   const int32_t* n_hits, int64_t B, float* out, float* out_q, float* out_pool, cudaStream_t st, const int64_t* offs);
 
 // transformer.cu: the Transformer in one kernel, likewise
 struct tf_tr_state;
 bool tf_tr_supported(const tf_shape& s);
 int tf_tr_create(trackfit_ctx* h, const float* host_w, tf_tr_state** out);
 void tf_tr_destroy(tf_tr_state* c);
-int tf_tr_forward(trackfit_ctx* h, tf_tr_state* c, uint64_t wait_ns, const float* hits, const int32_t* n_hits,
-                  int64_t B, float* out, float* out_q, float* out_pool, cudaStream_t st, const int64_t* offs);
+int tf_tr_forward(trackfit_ctx* h, tf_tr_state* c, uint64_t wait_ns, int hold_tile, const float* hits,
+                  const int32_t* n_hits, int64_t B, float* out, float* out_q, float* out_pool, cudaStream_t st, const int64_t* offs);
 
 // rows.cu
 bool tf_rows_supported(const tf_shape& s);
@@ -187,7 +187,7 @@ int tf_rows_create(trackfit_ctx* h, const float* host_w);
 void tf_rows_destroy(trackfit_ctx* h);
 int tf_rows_forward(trackfit_ctx* h, const float* hits, const int32_t* n_hits, int64_t B, float* out,
                     float* out_q, float* out_pool, cudaStream_t st, const int64_t* offs = nullptr);
-int tf_rows_wait_limit(trackfit_ctx* h, int64_t limit_ns);
+int tf_rows_wait_limit(trackfit_ctx* h, int64_t limit_ns, int hold_tile);
 
 // api.cu
 int tf_status_from_cuda(cudaError_t e);

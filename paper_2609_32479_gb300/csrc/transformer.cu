@@ -49,6 +49,7 @@ struct TrParams {
   const float* vec;             // b_e1, b_e2, then per layer g1, b_qkv, b_o, g2, b_1, b_2
   unsigned long long* err;
   uint64_t wait_ns;
+  int hold_tile;                // test hook: CTA 0's loader holds this tile's metadata hand-over (-1: none)
 };
 
 struct TrMisc {
@@ -374,7 +375,11 @@ __global__ void __launch_bounds__(NT, 1) transformer_kernel(const __grid_constan
     __syncwarp();
   } else if (warp < 2 + NE / 32) {
     // Epilogue.  A failed wait sets the abort flag and every later wait fails fast, but no
-    // warp leaves the loop early: all of them meet at the named barriers.
+    // warp leaves the loop early: all of them meet at the named barriers.  `alive` (the same
+    // for a warp's lanes): every wait of this warp has succeeded; only then is the metadata of
+    // its tile complete and kept until the warp releases it, and may an address be formed from
+    // it.
+    bool alive = true;
     const int q = warp & 3, cg = (warp - 2) >> 2, row = 32 * q + lane, c0 = 32 * cg;
     const int pair_bar = 1 + (q >> 1) * 4 + cg;   // 1-8: a slab's two quadrants, one column group
     const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16);
@@ -383,7 +388,10 @@ __global__ void __launch_bounds__(NT, 1) transformer_kernel(const __grid_constan
     uint32_t acc_k = 0, norms = 0;
     auto wait_on = [&](uint32_t bar, uint32_t parity) {
       const bool got = mbar_wait(bar, parity, abort, p.wait_ns);
-      if (!__all_sync(0xffffffffu, got) && lane == 0) tr_abort(m, p.err);
+      if (!__all_sync(0xffffffffu, got)) {
+        if (lane == 0) tr_abort(m, p.err);
+        alive = false;
+      }
       tc_fence_after();
     };
     auto wait_acc = [&]() { wait_on(acc_bar, acc_k++ & 1u); };
@@ -454,7 +462,7 @@ __global__ void __launch_bounds__(NT, 1) transformer_kernel(const __grid_constan
       wait_on(smem_u32(&m->meta_full[i & 1]), (uint32_t)(i >> 1) & 1u);
       const TileMeta* md = &m->meta[i & 1];
       int n = 0, start = row;
-      if (!*abort && (md->col_flags[row] & F_VALID)) {
+      if (alive && (md->col_flags[row] & F_VALID)) {
         n = md->slot_n[md->col_slot[row]];
         start = row - m->tpos[i & 1][row];
       }
@@ -494,7 +502,7 @@ __global__ void __launch_bounds__(NT, 1) transformer_kernel(const __grid_constan
       }
       // mean pooling, each track's hits in order: thread (track of the tile, channel)
       named_sync(13, NE);
-      if (!*abort) {
+      if (alive) {
         const int te = threadIdx.x - 64, c = te & 127;
         for (int w = 0; w < 4; ++w)   // tracks by their first row, in turn over the four thread groups
           for (uint32_t f = md->m_first[w >> 1][w & 1]; f; f &= f - 1) {
@@ -516,9 +524,14 @@ __global__ void __launch_bounds__(NT, 1) transformer_kernel(const __grid_constan
       if (i >= 2) {
         const bool got = mbar_wait(smem_u32(&m->meta_free[b]), (uint32_t)((i >> 1) - 1) & 1u, abort, p.wait_ns);
         if (!__all_sync(0xffffffffu, got) && lane == 0) tr_abort(m, p.err);
+        // after a failure anywhere a release may have come from a warp that gave up: stop, so
+        // that the metadata others still read stays as it is
+        if (!__all_sync(0xffffffffu, got && !*abort)) break;
       }
       load_meta(p.src, m->tpos[b], &m->meta[b], 2 * t, n_slabs, lane);
       __threadfence_block();
+      __syncwarp();
+      if (i == p.hold_tile && blockIdx.x == 0) hold_hand_over(abort, p.wait_ns);
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&m->meta_full[b]));
     }
@@ -666,12 +679,13 @@ int tf_tr_create(trackfit_ctx* h, const float* W, tf_tr_state** out) {
   return TRACKFIT_OK;
 }
 
-int tf_tr_forward(trackfit_ctx* h, tf_tr_state* c, uint64_t wait_ns, const float* hits, const int32_t* n_hits,
-                  int64_t B, float* out, float* out_q, float* out_pool, cudaStream_t st, const int64_t* offs) {
+int tf_tr_forward(trackfit_ctx* h, tf_tr_state* c, uint64_t wait_ns, int hold_tile, const float* hits,
+                  const int32_t* n_hits, int64_t B, float* out, float* out_q, float* out_pool, cudaStream_t st, const int64_t* offs) {
   const tf_shape& s = h->s;
   TrParams p = c->p;
   p.err = h->d_err;
   p.wait_ns = wait_ns;
+  p.hold_tile = hold_tile;
   const tf_pack pk = tf_pack_in(c->pack, c->chunk);
   p.src.T = s.T;
   p.src.slab = pk.slab;

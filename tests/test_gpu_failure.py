@@ -133,3 +133,45 @@ def test_failed_staging_allocation_in_forward_host_returns_oom(T):
         tf.forward_host(tb.hits, tb.n_hits, out)     # and then it works
         assert np.all(np.isfinite(out))
         assert T.debug_alloc(0)[0] == live0 + 3
+
+
+@pytest.mark.parametrize("name,n,tile", [("paper", 5000, 0), ("paper", 8000, 3), ("transformer", 5000, 0),
+                                         ("transformer", 8000, 3), ("medium", 8000, 3), ("large", 8000, 3)])
+def test_expired_wait_of_every_fused_kernel(T, name, n, tile):
+    """The same for the paper's model and the Transformer, and with a later tile held, when
+    the other warps are in mid-pipeline and earlier tiles' metadata is being reused."""
+    w = W.workload(name, n_tracks=n)
+    tb = W.gen_tracks(w)
+    dev = torch.device("cuda:0")
+    rows = W.paper_hits(tb, w) if w.model.n_features > 5 else tb.hits
+    hits, nh = torch.from_numpy(rows).to(dev), torch.from_numpy(tb.n_hits).to(dev)
+    out = torch.full((n, 5), -7.0, device=dev)
+    with T.Trackfit(w.model, W.gen_weights(w.model, w.weight_seed)) as tf:
+        tf.forward(hits, nh, out)
+        torch.cuda.synchronize()
+        assert tf.device_errors() == (T.OK, 0)
+        want = out.cpu().numpy()
+        tf.debug_wait_limit(50_000_000, hold_tile=tile)
+        t0 = time.perf_counter()
+        tf.forward(hits, nh, out)
+        torch.cuda.synchronize()
+        assert time.perf_counter() - t0 < 5.0
+        assert tf.device_errors()[0] == T.ERR_TIMEOUT
+        tf.debug_wait_limit(0, hold_tile=-1)
+        for _ in range(2):
+            out.fill_(-7.0)
+            tf.forward(hits, nh, out)
+            torch.cuda.synchronize()
+            assert tf.device_errors() == (T.OK, 0)
+            np.testing.assert_array_equal(out.cpu().numpy(), want)
+
+
+def test_hold_hook_is_refused_where_no_fused_kernel_runs(T):
+    m = W.workload("paper").model.with_(n_layers=3)
+    with T.Trackfit(m, W.gen_weights(m, 1)) as tf:
+        assert tf.path.startswith("tcgen05-rows")
+        tf.debug_wait_limit(1_000_000_000, -1)
+        for bad, status in (((-1, -1), T.ERR_INVALID_ARG), ((0, -2), T.ERR_INVALID_ARG), ((0, 0), T.ERR_UNSUPPORTED)):
+            with pytest.raises(T.TrackfitError) as ei:
+                tf.debug_wait_limit(*bad)
+            assert ei.value.status == status
