@@ -113,136 +113,136 @@ __global__ void __launch_bounds__(NT, 1) concat_kernel(const __grid_constant__ C
   volatile int* abort = &m->abort_flag;
 
   if (warp == 0) {
-    // TMA producer: the whole warp walks the blocks and waits; one lane's copies are let
-    // through by a predicate (see the issuer)
-    uint32_t stage = 0, phase = 0;
-    const uint32_t me = elect_one() ? 1u : 0u;
-    int issued = 0;
-    bool ok = true;
-    auto load = [&](int map, int c0, int c1) {
-      if (!ok) return;
-      const uint32_t full = full0 + 8 * stage;
-      if (!mbar_wait(empty0 + 8 * stage, phase ^ 1u, abort, p.wait_ns)) {
-        cat_abort(m, p.err);
-        ok = false;
-        return;
+    // TMA producer: one lane
+    if (elect_one()) {
+      uint32_t stage = 0, phase = 0;
+      int issued = 0;
+      bool ok = true;
+      auto load = [&](int map, int c0, int c1) {
+        if (!ok) return;
+        const uint32_t full = full0 + 8 * stage;
+        if (!mbar_wait(empty0 + 8 * stage, phase ^ 1u, abort, p.wait_ns)) {
+          cat_abort(m, p.err);
+          ok = false;
+          return;
+        }
+        mbar_arrive_expect_tx(full, A_BLOCK);
+        tma_load_2d(ring + stage * A_BLOCK, &p.tm[map], full, c0, c1);
+        ++issued;
+        if (++stage == (uint32_t)p.nst) {
+          stage = 0;
+          phase ^= 1u;
+        }
+      };
+      for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+        for (int kc = 0; kc < p.KE; ++kc) {
+          load(CM_E1, kc * 64, 0);
+          load(CM_F, kc * 64, t * TILE);
+        }
+        for (int kc = 0; kc < 2; ++kc) load(CM_E2, kc * 64, 0);
+        for (int l = 0; l < p.L; ++l)
+          for (int r = 0; r < 2 * CT_NDC; ++r)   // z, then n, of each chunk
+            for (int kc = 0; kc < (l ? 6 : 2); ++kc) load(l ? CM_IN1 : CM_IN0, kc * 64, r * 128);
       }
-      mbar_arrive_expect_tx_if(full, A_BLOCK, me);
-      tma_load_2d_if(ring + stage * A_BLOCK, &p.tm[map], full, c0, c1, me);
-      ++issued;
-      if (++stage == (uint32_t)p.nst) {
-        stage = 0;
-        phase ^= 1u;
+      if (*abort) {   // let the copies already issued land before the CTA can exit
+        volatile int never = 0;
+        for (int k = 0; k < p.nst && k < issued; ++k) {
+          const int i = issued - 1 - k;
+          mbar_wait(full0 + 8 * (i % p.nst), (uint32_t)((i / p.nst) & 1), &never, CT_DRAIN_NS);
+        }
       }
-    };
-    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
-      for (int kc = 0; kc < p.KE; ++kc) {
-        load(CM_E1, kc * 64, 0);
-        load(CM_F, kc * 64, t * TILE);
-      }
-      for (int kc = 0; kc < 2; ++kc) load(CM_E2, kc * 64, 0);
-      for (int l = 0; l < p.L; ++l)
-        for (int r = 0; r < 2 * CT_NDC; ++r)   // z, then n, of each chunk
-          for (int kc = 0; kc < (l ? 6 : 2); ++kc) load(l ? CM_IN1 : CM_IN0, kc * 64, r * 128);
     }
     __syncwarp();
-    if (*abort) {   // let the copies already issued land before the CTA can exit
-      volatile int never = 0;
-      for (int k = 0; k < p.nst && k < issued; ++k) {
-        const int i = issued - 1 - k;
-        mbar_wait(full0 + 8 * (i % p.nst), (uint32_t)((i / p.nst) & 1), &never, CT_DRAIN_NS);
-      }
-    }
   } else if (warp == 1) {
-    // MMA issuer: straight-line code for the whole warp, with the instructions of all
-    // lanes but one switched off by a predicate (an elected branch and a vote after each
-    // wait cost twice the time of the products)
-    uint32_t stage = 0, phase = 0, g = 0, op_k = 0;
-    const uint32_t me = elect_one() ? 1u : 0u;
-    bool ok = true;
-    auto wait_bar = [&](uint32_t bar, uint32_t parity) {
-      if (ok && !mbar_wait(bar, parity, abort, p.wait_ns)) {
-        cat_abort(m, p.err);
-        ok = false;
-      }
-    };
-    const uint64_t a_desc = sdesc_sw128(ring, 16, 1024), b_desc = sdesc_sw128(base, B_LBO, B_SBO);
-    const uint32_t a_lo0 = desc_lo(a_desc), a_hi = desc_hi(a_desc), b_lo0 = desc_lo(b_desc), b_hi = desc_hi(b_desc);
-    constexpr uint32_t BSTEP = (2 * B_SBO) >> 4;
-    auto stage_lo = [&]() { return a_lo0 + stage * (A_BLOCK >> 4); };
-    auto next_stage = [&]() {
-      if (++stage == (uint32_t)p.nst) {
-        stage = 0;
-        phase ^= 1u;
-      }
-    };
-    // the group's accumulator buffer, free once the epilogue has read group g - 2
-    auto begin = [&]() -> uint32_t {
-      if (g >= 2) wait_bar(acc_free + 8 * (g & 1u), ((g >> 1) - 1u) & 1u);
-      return tmem + (g & 1u) * 256u;
-    };
-    auto end = [&]() {
-      umma_commit_if(acc_full + 8 * (g & 1u), ok ? me : 0u);
-      ++g;
-    };
-    auto operand = [&]() { wait_bar(op_bar, op_k++ & 1u); };   // the epilogue's next operand hand-over
-    // kb (even) weight blocks against the activations at byte offset off of shared memory
-    auto product = [&](uint32_t d, uint32_t off, int kb) {
-      uint32_t b_lo = b_lo0 + (off >> 4);
-      for (int kc = 0; kc < kb; kc += 2, b_lo += 8 * BSTEP) {
-        wait_bar(full0 + 8 * stage, phase);
-        const uint32_t a0 = stage_lo(), e0 = empty0 + 8 * stage;
-        next_stage();
-        wait_bar(full0 + 8 * stage, phase);
-        if (!ok) return;
-        tc_fence_after();
-        umma4_f16_if<BSTEP>(d, a0, a_hi, b_lo, b_hi, p.idesc_mn, kc, me);
-        umma_commit_if(e0, me);
-        umma4_f16_if<BSTEP>(d, stage_lo(), a_hi, b_lo + 4 * BSTEP, b_hi, p.idesc_mn, 1u, me);
-        umma_commit_if(empty0 + 8 * stage, me);
-        next_stage();
-      }
-    };
-    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
-      {   // embedding product 1: weights and Fourier rows alternate in the ring
-        const uint32_t d = begin();
-        for (int kc = 0; kc < p.KE; ++kc) {
+    // MMA issuer: one lane for the whole loop (an elected branch and a vote at each wait
+    // cost twice the time of the products; the whole warp in step, as in tc_forward.cu, was
+    // 1 % slower here)
+    if (elect_one()) {
+      uint32_t stage = 0, phase = 0, g = 0, op_k = 0;
+      bool ok = true;
+      auto wait_bar = [&](uint32_t bar, uint32_t parity) {
+        if (ok && !mbar_wait(bar, parity, abort, p.wait_ns)) {
+          cat_abort(m, p.err);
+          ok = false;
+        }
+      };
+      const uint64_t a_desc = sdesc_sw128(ring, 16, 1024), b_desc = sdesc_sw128(base, B_LBO, B_SBO);
+      const uint32_t a_lo0 = desc_lo(a_desc), a_hi = desc_hi(a_desc), b_lo0 = desc_lo(b_desc), b_hi = desc_hi(b_desc);
+      constexpr uint32_t BSTEP = (2 * B_SBO) >> 4;
+      auto stage_lo = [&]() { return a_lo0 + stage * (A_BLOCK >> 4); };
+      auto next_stage = [&]() {
+        if (++stage == (uint32_t)p.nst) {
+          stage = 0;
+          phase ^= 1u;
+        }
+      };
+      // the group's accumulator buffer, free once the epilogue has read group g - 2
+      auto begin = [&]() -> uint32_t {
+        if (g >= 2) wait_bar(acc_free + 8 * (g & 1u), ((g >> 1) - 1u) & 1u);
+        return tmem + (g & 1u) * 256u;
+      };
+      auto end = [&]() {
+        if (ok) umma_commit(acc_full + 8 * (g & 1u));
+        ++g;
+      };
+      auto operand = [&]() { wait_bar(op_bar, op_k++ & 1u); };   // the epilogue's next operand hand-over
+      // kb (even) weight blocks against the activations at byte offset off of shared memory
+      auto product = [&](uint32_t d, uint32_t off, int kb) {
+        uint32_t b_lo = b_lo0 + (off >> 4);
+        for (int kc = 0; kc < kb; kc += 2, b_lo += 8 * BSTEP) {
           wait_bar(full0 + 8 * stage, phase);
           const uint32_t a0 = stage_lo(), e0 = empty0 + 8 * stage;
           next_stage();
           wait_bar(full0 + 8 * stage, phase);
-          if (!ok) break;
+          if (!ok) return;
           tc_fence_after();
-          if (kc + 1 < p.KE || p.last_nk == 4)
-            umma4_f16_if<2>(d, a0, a_hi, stage_lo(), a_hi, p.idesc_k, kc, me);
-          else
-            umma2_f16_if<2>(d, a0, a_hi, stage_lo(), a_hi, p.idesc_k, kc, me);
-          umma_commit_if(e0, me);
-          umma_commit_if(empty0 + 8 * stage, me);
+          umma4_f16<BSTEP>(d, a0, a_hi, b_lo, b_hi, p.idesc_mn, kc);
+          umma_commit(e0);
+          umma4_f16<BSTEP>(d, stage_lo(), a_hi, b_lo + 4 * BSTEP, b_hi, p.idesc_mn, 1u);
+          umma_commit(empty0 + 8 * stage);
           next_stage();
         }
-        end();
-      }
-      {   // embedding product 2 from the hidden values (Y's first rows)
-        const uint32_t d = begin();
-        operand();
-        product(d, CT_Y, 2);
-        end();
-      }
-      for (int l = 0; l < p.L && ok; ++l)
-        for (int dc = 0; dc < CT_NDC; ++dc) {
+      };
+      for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+        {   // embedding product 1: weights and Fourier rows alternate in the ring
           const uint32_t d = begin();
-          if (dc == 0) operand();
-          product(d, l ? CT_Y : CT_X, l ? 6 : 2);
-          product(d + 128, l ? CT_Y : CT_X, l ? 6 : 2);
+          for (int kc = 0; kc < p.KE; ++kc) {
+            wait_bar(full0 + 8 * stage, phase);
+            const uint32_t a0 = stage_lo(), e0 = empty0 + 8 * stage;
+            next_stage();
+            wait_bar(full0 + 8 * stage, phase);
+            if (!ok) break;
+            tc_fence_after();
+            if (kc + 1 < p.KE || p.last_nk == 4)
+              umma4_f16<2>(d, a0, a_hi, stage_lo(), a_hi, p.idesc_k, kc);
+            else
+              umma2_f16<2>(d, a0, a_hi, stage_lo(), a_hi, p.idesc_k, kc);
+            umma_commit(e0);
+            umma_commit(empty0 + 8 * stage);
+            next_stage();
+          }
           end();
         }
+        {   // embedding product 2 from the hidden values (Y's first rows)
+          const uint32_t d = begin();
+          operand();
+          product(d, CT_Y, 2);
+          end();
+        }
+        for (int l = 0; l < p.L && ok; ++l)
+          for (int dc = 0; dc < CT_NDC; ++dc) {
+            const uint32_t d = begin();
+            if (dc == 0) operand();
+            product(d, l ? CT_Y : CT_X, l ? 6 : 2);
+            product(d + 128, l ? CT_Y : CT_X, l ? 6 : 2);
+            end();
+          }
+      }
+      // no MMA may still run when TMEM is released
+      umma_commit(drain_bar);
+      volatile int never = 0;
+      mbar_wait(drain_bar, 0, &never, CT_DRAIN_NS);
     }
-    __syncwarp();
-    // no MMA may still run when TMEM is released (by the lane that issued them)
-    umma_commit_if(drain_bar, me);
-    volatile int never = 0;
-    mbar_wait(drain_bar, 0, &never, CT_DRAIN_NS);
     __syncwarp();
   } else if (warp < 2 + NE / 32) {
     // Epilogue.  The warps run decoupled: each arrives on the hand-over barriers itself

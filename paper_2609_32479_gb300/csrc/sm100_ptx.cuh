@@ -177,15 +177,6 @@ __device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t a_desc, uint6
       "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// As umma_f16, issued only if `issue` is nonzero (a guard predicate).
-__device__ __forceinline__ void umma_f16_if(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                            uint32_t accumulate, uint32_t issue) {
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
-      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(issue)
-      : "memory");
-}
 // Four MMAs of K = 16 over one 64-k block, issued only if `issue` is nonzero (a guard
 // predicate: the lanes of a converged warp but the elected one skip them without a
 // branch).  The descriptors come as halves; a step of K adds 2 to the low half of a
@@ -222,6 +213,16 @@ __device__ __forceinline__ void umma2_f16_if(uint32_t d_tmem, uint32_t a_lo, uin
       "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}" ::"r"(d_tmem),
       "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate), "r"(issue), "n"(BSTEP)
       : "memory");
+}
+template <int BSTEP>
+__device__ __forceinline__ void umma4_f16(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                          uint32_t idesc, uint32_t accumulate) {
+  umma4_f16_if<BSTEP>(d_tmem, a_lo, a_hi, b_lo, b_hi, idesc, accumulate, 1u);
+}
+template <int BSTEP>
+__device__ __forceinline__ void umma2_f16(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                          uint32_t idesc, uint32_t accumulate) {
+  umma2_f16_if<BSTEP>(d_tmem, a_lo, a_hi, b_lo, b_hi, idesc, accumulate, 1u);
 }
 // Arrive once on an mbarrier when all previously issued tcgen05.mma of this thread complete.
 __device__ __forceinline__ void umma_commit(uint32_t bar) {

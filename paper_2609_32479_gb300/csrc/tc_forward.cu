@@ -277,8 +277,9 @@ __global__ void __launch_bounds__(NT, 1) tc_forward_kernel(const __grid_constant
         if (!mbar_wait(empty0 + 8 * stage, phase ^ 1u, abort, p.wait_ns)) {
           set_abort(&m->abort_flag, p.err);
           ok = false;
-          break;
         }
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
         mbar_arrive_expect_tx_if(full, A_STAGE, me);
         tma_load_2d_if(dst, map, full, c0, c1, me);
         tma_load_2d_if(dst + A_BLOCK, map, full, tail ? c0 : c0 + 64, tail ? c1 + 128 : c1, me);
@@ -305,7 +306,10 @@ __global__ void __launch_bounds__(NT, 1) tc_forward_kernel(const __grid_constant
     // products beside busy warps (N = 64 products took as long as N = 128).  So the whole
     // warp runs one straight line a step, the instructions of all lanes but one are
     // switched off by a predicate, and the next step's entry is loaded ahead: 314
-    // cycles for 4.
+    // cycles for 4.  Every lane waits for itself, so the lanes vote once a step: one left
+    // behind by the length of the ring would test a parity two phases old (the vote takes
+    // 0.5 to 1 %; one lane alone for the whole loop took 3.47 ms instead of 3.26 for 20,011
+    // tracks).
     uint32_t stage = 0, phase = 0, e_k = 0, h_k = 0, a_k = 0;
     const uint32_t me = elect_one() ? 1u : 0u;
     bool ok = true;
@@ -331,6 +335,7 @@ __global__ void __launch_bounds__(NT, 1) tc_forward_kernel(const __grid_constant
           ++h_k;
         }
         wait_bar(full0 + 8 * stage, phase);
+        ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         tc_fence_after();
         const uint32_t a_lo = a_lo0 + stage * (A_STAGE >> 4), b_lo = b_lo0 + (e & 0xFFFFu);

@@ -168,8 +168,9 @@ __global__ void __launch_bounds__(PAIR_NT<THIN>, 1) tc_pair_kernel(const __grid_
           if (!mbar_wait(empty0 + 8 * stage, phase ^ 1u, abort, p.wait_ns)) {
             set_abort(&m->abort_flag, p.err);
             ok = false;
-            break;
           }
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
           mbar_arrive_expect_tx_if(full, A_BLOCK, me);
           tma_load_2d_if(ab + stage * A_BLOCK, map, full, c0, c1, me);
           ++issued;
@@ -189,7 +190,7 @@ __global__ void __launch_bounds__(PAIR_NT<THIN>, 1) tc_pair_kernel(const __grid_
       }
     }
   } else if (warp == 1) {
-    // MMA issuer: one straight line a step, as in the one-tile kernel
+    // MMA issuer: one straight line and one vote a step, as in the one-tile kernel
     uint32_t stage = 0, phase = 0;
     uint32_t e_k0 = 0, e_k1 = 0, h_k0 = 0, h_k1 = 0, a_k0 = 0, a_k1 = 0;   // hand-overs and commits so far, by tile
     const uint32_t me = elect_one() ? 1u : 0u;
@@ -226,10 +227,11 @@ __global__ void __launch_bounds__(PAIR_NT<THIN>, 1) tc_pair_kernel(const __grid_
           wait_bar(eh_bar + 8 * u, k & 1u);
         }
         wait_bar(full0 + 8 * stage, phase);
-        if (!ok) break;
         const uint32_t a_lo = a_lo0 + stage * (A_BLOCK >> 4), b_lo = b_lo0 + (e & 0xFFFFu);
         const uint32_t d = tmem + ((e & S_COL) >> 16) * 128u;
         if (e & S_TAIL) {
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
           tc_fence_after();
           umma2_f16_if<BSTEP>(d, a_lo, a_hi, b_lo, b_hi, idesc, 1u, me);
           umma_commit_if(empty0 + 8 * stage, me);
@@ -240,6 +242,7 @@ __global__ void __launch_bounds__(PAIR_NT<THIN>, 1) tc_pair_kernel(const __grid_
             phase ^= 1u;
           }
           wait_bar(full0 + 8 * stage, phase);
+          ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           tc_fence_after();
           umma4_f16_if<BSTEP>(d, a_lo, a_hi, b_lo, b_hi, idesc, e & S_ACC, me);

@@ -247,131 +247,133 @@ __global__ void __launch_bounds__(NT, 1) transformer_kernel(const __grid_constan
   const int kh = (p.H + 63) / 64;   // 64-k blocks of the hidden operand
 
   if (warp == 0) {
-    // TMA producer: blocks in the issuer's order, one lane's copies let through by a predicate
-    uint32_t stage = 0, phase = 0;
-    const uint32_t me = elect_one() ? 1u : 0u;
-    int issued = 0;
-    bool ok = true;
-    auto load = [&](int map, int c0, int c1, uint32_t bytes) {
-      if (!ok) return;
-      const uint32_t full = full0 + 8 * stage;
-      if (!mbar_wait(empty0 + 8 * stage, phase ^ 1u, abort, p.wait_ns)) {
-        tr_abort(m, p.err);
-        ok = false;
-        return;
+    // TMA producer: one lane, blocks in the issuer's order
+    if (elect_one()) {
+      uint32_t stage = 0, phase = 0;
+      int issued = 0;
+      bool ok = true;
+      auto load = [&](int map, int c0, int c1, uint32_t bytes) {
+        if (!ok) return;
+        const uint32_t full = full0 + 8 * stage;
+        if (!mbar_wait(empty0 + 8 * stage, phase ^ 1u, abort, p.wait_ns)) {
+          tr_abort(m, p.err);
+          ok = false;
+          return;
+        }
+        mbar_arrive_expect_tx(full, bytes);
+        tma_load_2d(ring + stage * A_BLOCK, &p.tm[map], full, c0, c1);
+        ++issued;
+        if (++stage == (uint32_t)p.nst) {
+          stage = 0;
+          phase ^= 1u;
+        }
+      };
+      for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+        for (int kc = 0; kc < p.KE; ++kc) {
+          load(TM_F, kc * 64, t * TILE, A_BLOCK);
+          load(TM_E1, kc * 64, 0, A_BLOCK);
+        }
+        for (int kc = 0; kc < 2; ++kc) load(TM_E2, kc * 64, 0, A_BLOCK);
+        for (int l = 0; l < p.L; ++l) {
+          for (int r = 0; r < 3; ++r)
+            for (int kc = 0; kc < 2; ++kc) load(TM_QKV, kc * 64, (3 * l + r) * 128, A_BLOCK);
+          for (int kc = 0; kc < 2; ++kc) load(TM_O, kc * 64, l * 128, A_BLOCK);
+          for (int r = 0; r < p.n1_tiles; ++r)
+            for (int kc = 0; kc < 2; ++kc) load(TM_1, kc * 64, l * p.H + r * p.n1, (uint32_t)p.n1 * 128u);
+          for (int kc = 0; kc < kh; ++kc) load(TM_2, kc * 64, l * 128, A_BLOCK);
+        }
       }
-      mbar_arrive_expect_tx_if(full, bytes, me);
-      tma_load_2d_if(ring + stage * A_BLOCK, &p.tm[map], full, c0, c1, me);
-      ++issued;
-      if (++stage == (uint32_t)p.nst) {
-        stage = 0;
-        phase ^= 1u;
-      }
-    };
-    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
-      for (int kc = 0; kc < p.KE; ++kc) {
-        load(TM_F, kc * 64, t * TILE, A_BLOCK);
-        load(TM_E1, kc * 64, 0, A_BLOCK);
-      }
-      for (int kc = 0; kc < 2; ++kc) load(TM_E2, kc * 64, 0, A_BLOCK);
-      for (int l = 0; l < p.L; ++l) {
-        for (int r = 0; r < 3; ++r)
-          for (int kc = 0; kc < 2; ++kc) load(TM_QKV, kc * 64, (3 * l + r) * 128, A_BLOCK);
-        for (int kc = 0; kc < 2; ++kc) load(TM_O, kc * 64, l * 128, A_BLOCK);
-        for (int r = 0; r < p.n1_tiles; ++r)
-          for (int kc = 0; kc < 2; ++kc) load(TM_1, kc * 64, l * p.H + r * p.n1, (uint32_t)p.n1 * 128u);
-        for (int kc = 0; kc < kh; ++kc) load(TM_2, kc * 64, l * 128, A_BLOCK);
+      if (*abort) {   // let the copies already issued land before the CTA can exit
+        volatile int never = 0;
+        for (int k = 0; k < p.nst && k < issued; ++k) {
+          const int i = issued - 1 - k;
+          mbar_wait(full0 + 8 * (i % p.nst), (uint32_t)((i / p.nst) & 1), &never, TR_DRAIN_NS);
+        }
       }
     }
     __syncwarp();
-    if (*abort) {   // let the copies already issued land before the CTA can exit
-      volatile int never = 0;
-      for (int k = 0; k < p.nst && k < issued; ++k) {
-        const int i = issued - 1 - k;
-        mbar_wait(full0 + 8 * (i % p.nst), (uint32_t)((i / p.nst) & 1), &never, TR_DRAIN_NS);
-      }
-    }
   } else if (warp == 1) {
-    // MMA issuer: straight-line code for the whole warp, all lanes but one switched off by
-    // a predicate.  Activations are the A operand, weights B, both K-major.
-    uint32_t stage = 0, phase = 0, op_k = 0;
-    const uint32_t me = elect_one() ? 1u : 0u;
-    bool ok = true;
-    auto wait_bar = [&](uint32_t bar, uint32_t parity) {
-      if (ok && !mbar_wait(bar, parity, abort, p.wait_ns)) {
-        tr_abort(m, p.err);
-        ok = false;
-      }
-    };
-    const uint64_t desc = sdesc_sw128(base, 16, 1024);
-    const uint32_t lo0 = desc_lo(desc), hi = desc_hi(desc), ring_lo = lo0 + (TR_RING >> 4);
-    auto stage_lo = [&]() { return ring_lo + stage * (A_BLOCK >> 4); };
-    auto next_stage = [&]() {
-      if (++stage == (uint32_t)p.nst) {
-        stage = 0;
-        phase ^= 1u;
-      }
-    };
-    auto operand = [&]() { wait_bar(op_bar, op_k++ & 1u); };   // the epilogue's next hand-over
-    auto commit = [&]() { umma_commit_if(acc_bar, ok ? me : 0u); };
-    // K columns of the operand at byte offset off, against the next blocks of the ring
-    auto product = [&](uint32_t d, uint32_t off, int K, uint32_t idesc) {
-      uint32_t a_lo = lo0 + (off >> 4);
-      for (int k = 0; k < K; k += 64, a_lo += A_BLOCK >> 4) {
-        wait_bar(full0 + 8 * stage, phase);
-        if (!ok) return;
-        tc_fence_after();
-        if (K - k >= 64) {
-          umma4_f16_if<2>(d, a_lo, hi, stage_lo(), hi, idesc, k, me);
-        } else {
-          for (int j = 0; j < (K - k) / 16; ++j)
-            umma_f16_if(d, ((uint64_t)hi << 32) | (a_lo + 2 * j), ((uint64_t)hi << 32) | (stage_lo() + 2 * j), idesc,
-                        (k | j) ? 1u : 0u, me);
+    // MMA issuer: one lane for the whole loop.  Activations are the A operand, weights B,
+    // both K-major.
+    if (elect_one()) {
+      uint32_t stage = 0, phase = 0, op_k = 0;
+      bool ok = true;
+      auto wait_bar = [&](uint32_t bar, uint32_t parity) {
+        if (ok && !mbar_wait(bar, parity, abort, p.wait_ns)) {
+          tr_abort(m, p.err);
+          ok = false;
         }
-        umma_commit_if(empty0 + 8 * stage, me);
-        next_stage();
-      }
-    };
-    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
-      if (t != (int)blockIdx.x) operand();   // the tile before has left the accumulators
-      for (int kc = 0; kc < p.KE; ++kc) {    // embedding product 1: Fourier rows and weights alternate in the ring
-        wait_bar(full0 + 8 * stage, phase);
-        const uint32_t a0 = stage_lo(), e0 = empty0 + 8 * stage;
-        next_stage();
-        wait_bar(full0 + 8 * stage, phase);
-        if (!ok) break;
-        tc_fence_after();
-        if (kc + 1 < p.KE || p.last_nk == 4)
-          umma4_f16_if<2>(tmem + 128, a0, hi, stage_lo(), hi, p.idesc, kc, me);
-        else
-          umma2_f16_if<2>(tmem + 128, a0, hi, stage_lo(), hi, p.idesc, kc, me);
-        umma_commit_if(e0, me);
-        umma_commit_if(empty0 + 8 * stage, me);
-        next_stage();
-      }
-      commit();
-      operand();
-      product(tmem + 128, TR_SA, 128, p.idesc);
-      commit();
-      for (int l = 0; l < p.L && ok; ++l) {
-        operand();
-        for (int r = 0; r < 3; ++r) product(tmem + 128 + 128 * r, TR_SA, 128, p.idesc);
+      };
+      const uint64_t desc = sdesc_sw128(base, 16, 1024);
+      const uint32_t lo0 = desc_lo(desc), hi = desc_hi(desc), ring_lo = lo0 + (TR_RING >> 4);
+      auto stage_lo = [&]() { return ring_lo + stage * (A_BLOCK >> 4); };
+      auto next_stage = [&]() {
+        if (++stage == (uint32_t)p.nst) {
+          stage = 0;
+          phase ^= 1u;
+        }
+      };
+      auto operand = [&]() { wait_bar(op_bar, op_k++ & 1u); };   // the epilogue's next hand-over
+      auto commit = [&]() { if (ok) umma_commit(acc_bar); };
+      // K columns of the operand at byte offset off, against the next blocks of the ring
+      auto product = [&](uint32_t d, uint32_t off, int K, uint32_t idesc) {
+        uint32_t a_lo = lo0 + (off >> 4);
+        for (int k = 0; k < K; k += 64, a_lo += A_BLOCK >> 4) {
+          wait_bar(full0 + 8 * stage, phase);
+          if (!ok) return;
+          tc_fence_after();
+          if (K - k >= 64) {
+            umma4_f16<2>(d, a_lo, hi, stage_lo(), hi, idesc, k);
+          } else {
+            for (int j = 0; j < (K - k) / 16; ++j)
+              umma_f16(d, ((uint64_t)hi << 32) | (a_lo + 2 * j), ((uint64_t)hi << 32) | (stage_lo() + 2 * j), idesc,
+                          (k | j) ? 1u : 0u);
+          }
+          umma_commit(empty0 + 8 * stage);
+          next_stage();
+        }
+      };
+      for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+        if (t != (int)blockIdx.x) operand();   // the tile before has left the accumulators
+        for (int kc = 0; kc < p.KE; ++kc) {    // embedding product 1: Fourier rows and weights alternate in the ring
+          wait_bar(full0 + 8 * stage, phase);
+          const uint32_t a0 = stage_lo(), e0 = empty0 + 8 * stage;
+          next_stage();
+          wait_bar(full0 + 8 * stage, phase);
+          if (!ok) break;
+          tc_fence_after();
+          if (kc + 1 < p.KE || p.last_nk == 4)
+            umma4_f16<2>(tmem + 128, a0, hi, stage_lo(), hi, p.idesc, kc);
+          else
+            umma2_f16<2>(tmem + 128, a0, hi, stage_lo(), hi, p.idesc, kc);
+          umma_commit(e0);
+          umma_commit(empty0 + 8 * stage);
+          next_stage();
+        }
         commit();
         operand();
         product(tmem + 128, TR_SA, 128, p.idesc);
         commit();
-        operand();
-        for (int r = 0; r < p.n1_tiles; ++r) product(tmem + 128 + (uint32_t)(r * p.n1), TR_SA, 128, p.idesc1);
-        commit();
-        operand();
-        product(tmem + 128, TR_KV, p.H, p.idesc);
-        commit();
+        for (int l = 0; l < p.L && ok; ++l) {
+          operand();
+          for (int r = 0; r < 3; ++r) product(tmem + 128 + 128 * r, TR_SA, 128, p.idesc);
+          commit();
+          operand();
+          product(tmem + 128, TR_SA, 128, p.idesc);
+          commit();
+          operand();
+          for (int r = 0; r < p.n1_tiles; ++r) product(tmem + 128 + (uint32_t)(r * p.n1), TR_SA, 128, p.idesc1);
+          commit();
+          operand();
+          product(tmem + 128, TR_KV, p.H, p.idesc);
+          commit();
+        }
       }
+      // no MMA may still run when TMEM is released
+      umma_commit(drain_bar);
+      volatile int never = 0;
+      mbar_wait(drain_bar, 0, &never, TR_DRAIN_NS);
     }
-    __syncwarp();
-    umma_commit_if(drain_bar, me);   // no MMA may still run when TMEM is released
-    volatile int never = 0;
-    mbar_wait(drain_bar, 0, &never, TR_DRAIN_NS);
     __syncwarp();
   } else if (warp < 2 + NE / 32) {
     // Epilogue.  A failed wait sets the abort flag and every later wait fails fast, but no
