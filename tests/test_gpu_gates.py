@@ -74,3 +74,17 @@ def test_a_gate_argument_that_is_not_a_number_shows(T, kind, row):
     m, w, h, nh = case(kind)
     w["layer0.b_in"][5 if row == "z" else 4 * m.d_hidden + 5] = np.nan
     assert not np.isfinite(run(T, m, w, h, nh)).any()
+
+
+@pytest.mark.parametrize("kind,n", [(MERGE128, 300), (MERGE128, 3000), (MERGE256, 300), (MERGE256, 3000)])
+def test_a_track_with_infinite_hits_leaves_the_others_alone(T, kind, n):
+    """One-slab tiles and pairs of tiles at d_model 128, one tile at 256: a track whose valid
+    hits hold infinities or NaN spoils its own row only, bit for bit."""
+    m, w, h, nh = case(kind, n)
+    want = run(T, m, w, h, nh)
+    h[17, : nh[17]] = np.inf
+    h[140, 0, 2] = np.nan
+    got = run(T, m, w, h, nh)
+    assert not np.isfinite(got[[17, 140]]).any()
+    others = np.setdiff1d(np.arange(n), [17, 140])
+    np.testing.assert_array_equal(got[others], want[others])
