@@ -404,10 +404,13 @@ extern "C" int trackfit_forward_host(trackfit_t h, const float* hits_host, const
   }
   cudaStream_t cs = h->cp_stream;
   cudaEvent_t* ev = h->cp_ev;
-  // Only the first step's copy is not hidden, so that step is short: its copy takes 0.08 ms
-  // instead of 0.6 ms at 24 hits a track (300,001 tracks of d_model 256: see the header for
-  // the steps).
-  const int64_t chunk = TF_HOST_CHUNK, head = n_tracks < TF_HOST_FIRST ? n_tracks : TF_HOST_FIRST;
+  // Only the first step's copy is not hidden, so that step is short where that saves more
+  // copying than a further step costs (a tile's chain of steps and four launches).  Short
+  // against whole first step, five features and 24 hits, ms at d_model 128 (six layers) and
+  // 256 (eight): 33,000 tracks 1.81 / 1.78 and 5.49 / 5.40, 65,000 3.31 / 3.32 and 10.29 /
+  // 10.27, 130,000 6.32 / 6.48 and 20.04 / 20.15, 300,001 14.22 / 14.68 and 45.72 / 46.13.
+  const int64_t chunk = TF_HOST_CHUNK, first = n_tracks < TF_HOST_SPLIT ? chunk : TF_HOST_FIRST;
+  const int64_t head = n_tracks < first ? n_tracks : first;
   const int64_t n_chunks = 1 + (n_tracks - head + chunk - 1) / chunk;
   auto start = [&](int64_t k) { return k == 0 ? 0 : head + (k - 1) * chunk; };
   auto count = [&](int64_t k) {

@@ -25,7 +25,8 @@ struct tf_nvtx_range {
 #define TF_PACK_TRACKS 4194304  // tracks that a handle packs at a time
 #define TF_PACKED_CHUNK 1048576
 #define TF_HOST_FIRST 32768   // tracks of the first copy / compute step of trackfit_forward_host
-#define TF_HOST_CHUNK 262144  // tracks of the others
+#define TF_HOST_SPLIT 98304   // .. in batches of at least this many tracks
+#define TF_HOST_CHUNK 262144  // tracks of the other steps
 #define TF_HOST_EVENTS 10
 
 // Offsets (in floats) of every tensor inside the fp32 weight blob.

@@ -222,3 +222,23 @@ def test_hit_rows_of_fifteen_features_in_host_buffers_and_chunks(T):
     got, _ = forward(T, m, blob, hits[:5200], tb.n_hits[:5200])
     few, _ = forward(T, m, blob, hits[5000:5200], tb.n_hits[5000:5200])
     np.testing.assert_array_equal(got[5000:], few)
+
+
+@pytest.mark.parametrize("n,steps", [(33000, 1), (98303, 1), (98304, 2), (400000, 3)])
+def test_steps_of_a_host_batch(T, n, steps):
+    """A short first step only where it saves more copying than a further step costs (33,000
+    tracks in two steps took 2 % longer than in one), and the device's results bit for bit."""
+    w = W.workload("tiny" if n == 400000 else "paper", n_tracks=4000)
+    tb = W.gen_tracks(w)
+    rows = W.paper_hits(tb, w) if w.model.n_features > 5 else tb.hits
+    hits, nh = np.resize(rows, (n, *rows.shape[1:])), np.resize(tb.n_hits, n)
+    blob = W.gen_weights(w.model, 2)
+    want, _ = forward(T, w.model, blob, hits, nh)
+    out = np.full((n, 5), -7.0, np.float32)
+    with T.Trackfit(w.model, blob) as tf:
+        tf.profile(True)
+        tf.forward_host(hits, nh, out)
+        _, launches = tf.profile_read()
+        tf.profile(False)
+    assert launches == steps
+    np.testing.assert_array_equal(out, want)
