@@ -292,19 +292,31 @@ cudaError_t tf_fused_fp32_prepare(const tf_shape& s) {
 // can take its tracks whole at once (and in 16 rows if they fit), the batch goes out
 // as runs of consecutive tracks, without packing: its time is one CTA's chain of
 // steps then, which neither packing nor fuller CTAs would shorten.  Above that the
-// slabs of the packing keep 97 % of the rows busy.
+// slabs of the packing keep 97 % of the rows busy.  An SM has two slots, or one at d_model
+// 128 (by registers) and where shared memory holds only one CTA of 64 rows (d_model 80 up,
+// any with 15 features): with two assumed there, 304 tracks of 20 hits at d_model 96 ran
+// unpacked in two waves, more than 1.5 times the 226 us of one.
 int tf_fused_fp32_forward(const tf_shape& s, const tf_blob_off& o, const float* W, const tf_pack& pk,
                           unsigned long long* err, const float* hits, const int32_t* n_hits, const int64_t* offs,
                           int64_t B, float* out, float* out_q, float* out_pool, cudaStream_t st, trackfit_ctx* prof) {
-  int dev = 0, nsm = 0;
+  int dev = 0, nsm = 0, sm_smem = 0, reserved = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess)
     return TRACKFIT_ERR_CUDA;
+  const Plan q1 = shape_plan(s, 1), q4 = shape_plan(s, 4);
+  auto slots_of = [&](const Plan& q) -> int64_t {
+    const bool two = q.CP != 8 && 2 * (q.smem + sizeof(Meta) + reserved) <= (size_t)sm_smem;
+    return (int64_t)nsm * (two ? 2 : 1);
+  };
+  const int64_t slots1 = slots_of(q1), slots4 = slots_of(q4);
   for (int64_t c0 = 0; c0 < B; c0 += pk.cap) {
     const int64_t nb = B - c0 < pk.cap ? B - c0 : pk.cap;
-    const int64_t slots = (int64_t)nsm * (s.D == 128 ? 1 : 2), each = (nb + slots - 1) / slots;
-    const bool flat = each * s.T <= TF_SLAB && each <= TF_SLAB_TRACKS;
-    const Plan q = shape_plan(s, flat && each * s.T <= 16 ? 1 : 4);
+    const int64_t each1 = (nb + slots1 - 1) / slots1, each4 = (nb + slots4 - 1) / slots4;
+    const bool small = each1 * s.T <= 16, flat = small || (each4 * s.T <= TF_SLAB && each4 <= TF_SLAB_TRACKS);
+    const Plan& q = small ? q1 : q4;
+    const int64_t slots = small ? slots1 : slots4, each = small ? each1 : each4;
     FusedArgs p{s, o, W, offs ? hits : hits + c0 * s.T * s.F, offs ? offs + c0 : nullptr, n_hits + c0, nb,
                 flat ? (int)each : 0, pk.order, pk.slab, pk.n_slabs, q.ldx, q.ldy, q.ldr,
                 out + c0 * 5, out_q ? out_q + c0 * s.Q : nullptr, out_pool ? out_pool + c0 * s.P : nullptr, err};

@@ -242,3 +242,29 @@ def test_steps_of_a_host_batch(T, n, steps):
         tf.profile(False)
     assert launches == steps
     np.testing.assert_array_equal(out, want)
+
+
+@pytest.mark.parametrize("D,F", [(96, 5), (112, 5), (32, 15)])
+def test_fp32_batch_of_two_tracks_an_sm_takes_one_wave(T, D, F):
+    """Where one CTA of 64 rows fits an SM, twice as many tracks of 20 hits as SMs go two to
+    a CTA: about the time of one track to a CTA, where two waves take twice that."""
+    m = W.ModelConfig(max_hits=20, d_model=D, d_hidden=3 * D // 2, n_layers=2, n_features=F,
+                      feat_min=W.PAPER_FEAT_MIN[:F], feat_max=W.PAPER_FEAT_MAX[:F])
+    dev = torch.device("cuda:0")
+    nsm = torch.cuda.get_device_properties(dev).multi_processor_count
+    us = {}
+    with T.Trackfit(m, W.gen_weights(m, 2)) as tf:
+        for n in (nsm, 2 * nsm):
+            h, nh = torch.rand((n, 20, F), device=dev), torch.full((n,), 20, dtype=torch.int32, device=dev)
+            out, ts = torch.empty((n, 5), device=dev), []
+            for _ in range(20):
+                a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+                a.record()
+                for _ in range(10):
+                    tf.forward(h, nh, out)
+                b.record()
+                torch.cuda.synchronize()
+                ts.append(a.elapsed_time(b) * 100)
+            us[n] = min(ts)
+    print(D, F, us)
+    assert us[2 * nsm] < 1.5 * us[nsm], us
