@@ -10,12 +10,9 @@ namespace tf_ffma {
 constexpr int NTHREADS = 256;
 constexpr int KC = 16;   // k per staged weight chunk (every K of the encoder and the head is a multiple of 16)
 
-// sigma(x) = 1 / (1 + e^-x): the library exponential, the hardware reciprocal
-// refined once (e^-x = inf gives 0)
-__device__ __forceinline__ float sigm(float x) {
-  const float d = 1.0f + expf(-x);
-  return __fdividef(1.0f, d);
-}
+// sigma(x) = 1 / (1 + e^-x): the library exponential and the IEEE division (e^-x = inf
+// gives 0)
+__device__ __forceinline__ float sigm(float x) { return 1.0f / (1.0f + expf(-x)); }
 __device__ __forceinline__ float silu(float x) { return x * sigm(x); }
 
 // floats of the two staging buffers for CN columns a thread

@@ -268,3 +268,27 @@ def test_fp32_batch_of_two_tracks_an_sm_takes_one_wave(T, D, F):
             us[n] = min(ts)
     print(D, F, us)
     assert us[2 * nsm] < 1.5 * us[nsm], us
+
+
+@pytest.mark.parametrize("prec", [W.PRECISION_FP32, W.PRECISION_BF16])
+def test_sigmoid_of_the_fp32_parts_divides_exactly(T, prec):
+    """W_h1 = 0 and rows of W_h2 that pick one hidden value make the quantiles SiLU(b_h1): the
+    bits of x / (1 + e^-x) with fp32's own exponential, division and product, in the fp32
+    encoder's head and in the 16-bit paths'."""
+    m = W.ModelConfig(max_hits=8, d_model=128, d_hidden=192, n_layers=1, n_quantiles=15, precision=prec)
+    w = W.split_weights(m, W.gen_weights(m, 2))
+    w["head.w1"][:] = 0.0
+    w["head.w2"][:] = np.eye(75, 128, dtype=np.float32)
+    w["head.b2"][:] = 0.0
+    dev = torch.device("cuda:0")
+    h, nh = torch.rand((4, 8, 5), device=dev), torch.full((4,), 5, dtype=torch.int32, device=dev)
+    for seed in range(6):
+        x = np.random.default_rng(seed).uniform(-20.0, 20.0, 128).astype(np.float32)
+        w["head.b1"][:] = x
+        with T.Trackfit(m, W.join_weights(m, w)) as tf:
+            out, q = torch.empty((4, 5), device=dev), torch.empty((4, 5, 15), device=dev)
+            tf.forward(h, nh, out, quantiles=q)
+            torch.cuda.synchronize()
+        t = torch.from_numpy(x[:75]).to(dev)
+        want = t * (1.0 / (1.0 + torch.exp(-t)))
+        np.testing.assert_array_equal(q.reshape(4, 75).cpu().numpy(), np.broadcast_to(want.cpu().numpy(), (4, 75)))
