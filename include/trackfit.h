@@ -300,7 +300,8 @@ int trackfit_debug_umma(trackfit_t h, const uint16_t* A, const uint16_t* Bkn, in
  * asinh(dv) and s_helix, where the foot point is the helix point whose normal
  * plane holds the hit (Newton's method), du and dv the hit's coordinates there
  * along U = z x t / |z x t| and V = t x U (the curvilinear frame), s the 3-D
- * path length from the perigee, lengths in mm (asinh scale 1 mm).
+ * path length from the perigee, lengths in mm (asinh scale 1 mm); the fp64 values,
+ * asinh to 2e-12 of them, rounded to fp32.
  *   hits         device [n_tracks][max_hits][hit_stride] fp32, x, y, z [mm] first.
  *   hit_stride   floats per hit row (>= 3; 5 for the task's inputs, 15 for the paper's).
  *   n_hits       device [n_tracks] int32.

@@ -72,8 +72,8 @@ __device__ __forceinline__ double rcp_n(double v) {
 // asinh(x) = sign(x) log(1 + t), t = |x| + x^2 / (1 + sqrt(1 + x^2)), with
 // log(1 + t) = e log 2 + 2 atanh(r), r = (m - 1) / (m + 1) for 1 + t = m 2^e with
 // m in [1/sqrt 2, sqrt 2] (r = t / (2 + t) for small t, without forming 1 + t).
-// |r| < 0.172, so the series of atanh to r^13 leaves 5e-11 relative: far below the
-// fp32 rounding of the feature.
+// |r| < 0.172, so the series of atanh to r^13 leaves 1.3e-12 relative at most, the
+// reciprocals 4e-13 each: 3e-5 of the fp32 rounding of the feature.
 __device__ __forceinline__ double asinh_n(double x) {
   const double ax = fabs(x);
   if (!(ax < 1e9)) return asinh(x);
@@ -194,9 +194,12 @@ __device__ void perigee_from_triplet(const double (&a)[3], const double (&b)[3],
 //
 // The fp64 pipe bounds this.  So the angle is evaluated once: the sine and cosine of
 // the direction at the start are the hit's own unit vector from the centre, and each
-// step turns them by the small angle of the step.  g'' is the hit's distance from the
-// helix times sin(theta), so the error after a step d is at most d^2 times that
-// distance over 2 R: a step of 1e-5 is the last (it leaves 1e-10 of the distance in s).
+// step turns them by the small angle of the step.  g'' is sin^2(theta) times the distance w
+// of the hit from the foot point along the transverse direction, so the angle is off by at
+// most d^2 w / 2 |g'| after a step d: one of 1e-5 is the last if w is below |g'| / 500 (g' is
+// near R / sin(theta): hits within a millimetre or so; it leaves 1e-13), else one of 1e-8.
+// (With 1e-5 for every hit s was up to 5e-9 off for hits 100 mm beside the helix, 2e-8 at
+// 1 m, near fp32's rounding.)
 __device__ __forceinline__ void residuals(const Helix& h, double x, double y, double z, double& du, double& dv,
                                           double& s) {
   double hx = x - h.cx, hy = y - h.cy;
@@ -216,16 +219,16 @@ __device__ __forceinline__ void residuals(const Helix& h, double x, double y, do
     ry = y - (h.cy + qR * cphi);
     rz = z - fma(h.rcot, a, h.z0);
     if (it == NEWTON_MAX) break;
-    const double g = h.st * (rx * cphi + ry * sphi) + h.ct * rz;
+    const double w = rx * cphi + ry * sphi, g = h.st * w + h.ct * rz;
     // dp/da = (R / sin theta) t;  dt/da = q sin(theta) (sin phi, -cos phi, 0)
-    const double d = -g * rcp_n<1>(qst * (rx * sphi - ry * cphi) - h.r_st);
+    const double dg = qst * (rx * sphi - ry * cphi) - h.r_st, d = -g * rcp_n<1>(dg);
     a += d;
     double sd, cd;
     sincos_step(-h.q * d, sd, cd);   // phi = phi0 - q a
     const double s1 = sphi * cd + cphi * sd;
     cphi = cphi * cd - sphi * sd;
     sphi = s1;
-    if (fabs(d) <= 1e-5) it = NEWTON_MAX - 1;   // one more pass for the residual, then out
+    if (fabs(d) <= (500.0 * fabs(w) <= fabs(dg) ? 1e-5 : 1e-8)) it = NEWTON_MAX - 1;   // one more pass for the residual, then out
   }
   // U = (-sin phi, cos phi, 0); V = t x U = (-cos theta cos phi, -cos theta sin phi, sin theta)
   du = ry * cphi - rx * sphi;

@@ -292,3 +292,67 @@ def test_sigmoid_of_the_fp32_parts_divides_exactly(T, prec):
         t = torch.from_numpy(x[:75]).to(dev)
         want = t * (1.0 / (1.0 + torch.exp(-t)))
         np.testing.assert_array_equal(q.reshape(4, 75).cpu().numpy(), np.broadcast_to(want.cpu().numpy(), (4, 75)))
+
+
+@pytest.mark.parametrize("off", [30.0, 300.0])
+def test_seed_features_are_fp64_results_rounded_once(T, off):
+    """Hits moved off their tracks: the features are the fp64 oracle's rounded to fp32.  The two
+    sides' positions carry 2e-13 mm, 2e-13 of a residual of 1 mm or more, and the device's
+    asinh 2e-12, which straddle a rounding boundary (6e-8 apart) in fewer than 4e-5 of the
+    values; s has no asinh."""
+    n = 20000
+    w = W.Workload("t", n, W.workload("medium").model, layout="barrel", pt_range=(0.5, 2.0), min_hits=8)
+    tb = W.gen_tracks(w, seed=9)
+    T_ = tb.hits.shape[1]
+    rng = np.random.default_rng(4)
+    hits = tb.hits.copy()
+    hits[:, 5:, :3] += rng.uniform(-off, off, hits[:, 5:, :3].shape).astype(np.float32)
+    dev = torch.device("cuda:0")
+    h, nh = torch.from_numpy(hits).to(dev), torch.from_numpy(tb.n_hits).to(dev)
+    sd = torch.empty((n, 5), dtype=torch.float64, device=dev)
+    ft = torch.empty((n, T_, 3), device=dev)
+    T.seed(h, nh, 2.0, sd, ft)
+    feats = ft.cpu().numpy()
+    ref = S.seed_from_hits(hits, tb.n_hits, 2.0)
+    fref = S.seed_features(ref, hits, tb.n_hits, 2.0)
+    at = np.arange(T_)[None, :]
+    moved = (at < tb.n_hits[:, None]) & (at >= 5) & ~np.isnan(ref[:, :1])
+    got, want = feats[moved], fref[moved]
+    uv = np.abs(np.sinh(want[:, :2]))
+    near = (uv > 1.0).all(1) & (uv < 2.0 * off).all(1)
+    assert near.sum() > 50000
+    wrong = (got[near] != want[near].astype(np.float32)).mean(0)
+    print("share of values that differ:", wrong, "of", near.sum())
+    assert (wrong <= [4e-5, 4e-5, 2e-5]).all(), wrong
+
+
+def test_seed_search_goes_on_where_a_small_step_is_not_the_last(T):
+    """Hits up to 1.5 m beside the helix, of them those where stopping the foot point search
+    at the first step of 1e-5 rad or less leaves the path length off by a quarter of an fp32
+    spacing or more (from the oracle's own iterates): the feature is the converged value
+    rounded."""
+    n = 20000
+    w = W.Workload("t", n, W.workload("medium").model, layout="barrel", pt_range=(0.3, 2.0), min_hits=8)
+    tb = W.gen_tracks(w, seed=11)
+    hits = tb.hits.copy()
+    rng = np.random.default_rng(6)
+    hits[:, 5:, :3] += rng.uniform(-1500.0, 1500.0, hits[:, 5:, :3].shape).astype(np.float32)
+    ref = S.seed_from_hits(hits, tb.n_hits, 2.0)
+    at = np.arange(hits.shape[1])[None, :]
+    b, t = np.nonzero((at < tb.n_hits[:, None]) & (at >= 5) & np.isfinite(ref).all(1)[:, None])
+    pg, x = ref[b], hits[b, t, :3].astype(np.float64)
+    s = np.stack([S.curvilinear_residuals(pg, x, 2.0, iters=k)[2] for k in (0, 1, 2, 3, 4, 5, 6, 40)])
+    per_rad = 1000.0 / (np.abs(pg[:, 4]) * S.C_LIGHT * 2.0)
+    small = np.abs(np.diff(s[:7], axis=0)) / per_rad <= 1e-5
+    stop = np.where(small.any(0), small.argmax(0) + 1, 7)
+    left = np.abs(s[stop, np.arange(len(b))] - s[7])
+    hard = (left > 0.25 * np.spacing(np.abs(s[7]).astype(np.float32))) & (np.abs(s[6] - s[7]) < 1e-12 * np.abs(s[7]))
+    assert hard.sum() >= 2   # of 100,000: rare, and wrong in the last bit
+    dev = torch.device("cuda:0")
+    sd = torch.empty((n, 5), dtype=torch.float64, device=dev)
+    ft = torch.empty((*hits.shape[:2], 3), device=dev)
+    T.seed(torch.from_numpy(hits).to(dev), torch.from_numpy(tb.n_hits).to(dev), 2.0, sd, ft)
+    got = ft.cpu().numpy()[b, t, 2]
+    wrong = got[hard] != s[7][hard].astype(np.float32)
+    print("hard hits:", hard.sum(), "not the converged value:", wrong.sum())
+    assert wrong.sum() == 0
