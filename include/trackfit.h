@@ -264,17 +264,20 @@ int trackfit_debug_scan(const float* a, const float* b, const float* x, const in
                         int64_t n_tracks, int32_t T, int32_t C, float* h_fwd, float* h_bwd,
                         void* stream);
 
-/* Test hook, host only (no GPU needed): per-tile totals of the tensor-core
- * path's block schedule for cfg, from the same expansion the fused kernel uses.
- * counts (host, n_counts >= 6): [0] 128 x 64 weight blocks, [1] MMA instructions
- * (128 x 128 x 16 each), [2] operand hand-overs the issuer waits for from the
- * epilogue (W_E), [3] state hand-overs (W_H), [4] accumulator commits the
- * epilogue waits for (C_ACC), [5] state-buffer commits (C_HB).  codes (host,
+/* Test hook, host only (no GPU needed): totals of the tensor-core path's block
+ * schedules for cfg, from the same expansion the fused kernel uses.
+ * counts (host, n_counts >= 6), of a tile by itself: [0] 128 x 64 weight blocks, [1]
+ * MMA instructions (128 x 128 x 16 each), [2] operand hand-overs the issuer waits for
+ * from the epilogue (W_E), [3] state hand-overs (W_H), [4] accumulator commits the
+ * epilogue waits for (C_ACC), [5] state-buffer commits (C_HB); with n_counts >= 12,
+ * [6..11] the same of two tiles in turn (d_model 128; zeros else).  codes (host,
  * optional, NULL when codes_cap is 0): the first codes_cap blocks' hand-overs in
- * issue order, one byte each: wait (0 none, 1 W_E, 2 W_H) | commit (0 none,
- * 1 C_ACC, 2 C_HB) << 2.  Returns TRACKFIT_ERR_UNSUPPORTED when cfg does not run
- * on the tensor-core path, TRACKFIT_ERR_INVALID_ARG for NULL pointers, n_counts
- * < 6, or codes_cap > 0 with codes NULL. */
+ * issue order, one byte each: wait (0 none, 1 W_E, 2 W_H) | commit (0 none, 1 C_ACC,
+ * 2 C_HB) << 2; with n_counts >= 12 the two tiles' blocks follow, as waits (1 W_E, 2
+ * W_H, 4 an operand hand-over of the other tile) | commit << 3 | tile << 5.  Returns
+ * TRACKFIT_ERR_UNSUPPORTED when cfg does not run on the tensor-core path,
+ * TRACKFIT_ERR_INVALID_ARG for NULL pointers, n_counts < 6, or codes_cap > 0 with
+ * codes NULL. */
 int trackfit_debug_schedule(const trackfit_config_t* cfg, int64_t* counts, int32_t n_counts, uint8_t* codes,
                             int64_t codes_cap);
 

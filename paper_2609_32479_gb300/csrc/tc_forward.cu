@@ -749,30 +749,31 @@ static std::vector<Step> build_schedule(int D, int L, int NDC, int ROWS_IN, int 
   return out;
 }
 
-struct ScheduleCounter {   // a callable for walk_tile on either side
+struct ScheduleCounter {   // a callable for walk_tile and walk_pair on either side
   int64_t c[6] = {0, 0, 0, 0, 0, 0};
   uint8_t* codes = nullptr;   // optional: per block wait | commit << 2, in order
   int64_t cap = 0;
-  void operator()(int, int, int, int nk, int, int, int, int, int wait, int commit) {
-    if (c[0] < cap) codes[c[0]] = (uint8_t)(wait | (commit << 2));
+  bool two = false;           // two tiles in turn: wait | commit << 3 | tile << 5
+  void operator()(int u, int, int, int, int nk, int, int, int, int, int wait, int commit) {
+    if (c[0] < cap) codes[c[0]] = (uint8_t)(two ? wait | (commit << 3) | (u << 5) : wait | (commit << 2));
     ++c[0];
     c[1] += nk;
-    c[2] += wait == W_E;
-    c[3] += wait == W_H;
+    c[2] += ((wait & W_E) != 0) + ((wait & W_X) != 0);
+    c[3] += (wait & W_H) != 0;
     c[4] += commit == C_ACC;
     c[5] += commit == C_HB;
   }
-  void operator()(int, int map, int row, int col, int nk, int tcol, int bsel, int bk, int acc,
-                                      int wait, int commit) {   // walk_pair
-    (*this)(map, row, col, nk, tcol, bsel, bk, acc, wait, commit);
+  void operator()(int map, int row, int col, int nk, int tcol, int bsel, int bk, int acc, int wait, int commit) {
+    (*this)(0, map, row, col, nk, tcol, bsel, bk, acc, wait, commit);
   }
 };
 
-// Per-tile totals of the fused kernel's block schedule, from the same walk_tile
-// the kernel expands (host only, no device needed): counts[0] blocks, [1] MMA
-// instructions (128 x 128 x 16 each), [2] W_E and [3] W_H hand-over waits, [4]
-// C_ACC and [5] C_HB commits; with codes, also each block's wait | commit << 2
-// in issue order (at most cap blocks).
+// Totals of the fused kernel's block schedules, from the walks the kernel's steps are made
+// from (host only, no device needed): counts[0] blocks, [1] MMA instructions (128 x 128 x 16
+// each), [2] W_E and [3] W_H hand-over waits, [4] C_ACC and [5] C_HB commits of a tile by
+// itself; with n >= 12, [6..11] the same of two tiles in turn (d_model 128, else 0).  With
+// codes, also each block's waits and commit in issue order (at most cap blocks): the lone
+// tile's, then, with n >= 12, the two tiles'.
 int tf_tc_schedule_counts(const tf_shape& s, int64_t* counts, int n, uint8_t* codes, int64_t cap) {
   if (n < 6 || (cap > 0 && !codes)) return TRACKFIT_ERR_INVALID_ARG;
   TcParams q;
@@ -781,7 +782,7 @@ int tf_tc_schedule_counts(const tf_shape& s, int64_t* counts, int n, uint8_t* co
   q.L = s.L;
   q.NDC = s.H / 64;
   q.ROWS_IN = q.NDC * 256 + s.D;
-  ScheduleCounter c;
+  ScheduleCounter c, c2;
   c.codes = codes;
   c.cap = cap;
   if (s.D == 128)
@@ -789,6 +790,14 @@ int tf_tc_schedule_counts(const tf_shape& s, int64_t* counts, int n, uint8_t* co
   else
     walk_tile(q, c);
   for (int i = 0; i < 6; ++i) counts[i] = c.c[i];
+  if (n < 12) return TRACKFIT_OK;
+  c2.two = true;
+  if (cap > c.c[0]) {
+    c2.codes = codes + c.c[0];
+    c2.cap = cap - c.c[0];
+  }
+  if (s.D == 128) walk_pair(q.L, q.NDC, q.ROWS_IN, 2, c2);
+  for (int i = 0; i < 6; ++i) counts[6 + i] = c2.c[i];
   return TRACKFIT_OK;
 }
 

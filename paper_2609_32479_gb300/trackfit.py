@@ -136,25 +136,28 @@ def weight_count(m: W.ModelConfig) -> int:
     return int(load().trackfit_weight_count(ctypes.byref(c)))
 
 
-def schedule_counts(m: W.ModelConfig, with_codes: bool = False):
-    """Per-tile totals of the tensor-core path's block schedule (host only): dict
-    with blocks, mmas, w_e, w_h, c_acc, c_hb (and, with_codes, "codes": each block's
-    wait | commit << 2 in issue order); None when m does not run on that path."""
+def schedule_counts(m: W.ModelConfig, with_codes: bool = False, two: bool = False):
+    """Totals of the tensor-core path's block schedule (host only) for a tile by itself or,
+    with two, for two tiles in turn: dict with blocks, mmas, w_e, w_h, c_acc, c_hb (and,
+    with_codes, "codes": each block's wait | commit << 2 in issue order, with two its waits
+    | commit << 3 | tile << 5); None when m does not run on that path."""
     c = make_config(m)
-    out = (ctypes.c_int64 * 6)()
+    out = (ctypes.c_int64 * 12)()
     lib = load()
-    st = lib.trackfit_debug_schedule(ctypes.byref(c), out, 6, None, 0)
+    st = lib.trackfit_debug_schedule(ctypes.byref(c), out, 12, None, 0)
     if st == ERR_UNSUPPORTED:
         return None
     if st != OK:
         raise TrackfitError(st, "trackfit_debug_schedule")
-    res = dict(zip(("blocks", "mmas", "w_e", "w_h", "c_acc", "c_hb"), (int(v) for v in out)))
+    counts = [int(v) for v in out]
+    res = dict(zip(("blocks", "mmas", "w_e", "w_h", "c_acc", "c_hb"), counts[6:] if two else counts[:6]))
     if with_codes:
-        codes = (ctypes.c_uint8 * res["blocks"])()
-        st = lib.trackfit_debug_schedule(ctypes.byref(c), out, 6, codes, res["blocks"])
+        n = counts[0] + counts[6]
+        codes = (ctypes.c_uint8 * n)()
+        st = lib.trackfit_debug_schedule(ctypes.byref(c), out, 12, codes, n)
         if st != OK:
             raise TrackfitError(st, "trackfit_debug_schedule")
-        res["codes"] = list(codes)
+        res["codes"] = list(codes)[counts[0]:] if two else list(codes)[:counts[0]]
     return res
 
 

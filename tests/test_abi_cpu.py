@@ -233,3 +233,106 @@ def test_no_epilogue_warp_falls_two_commits_behind(lib, D, H, L):
                 assert gate >= j - 1, f"commit {j} can land while a warp still waits for commit {j - 2}"
             j += 1
     assert n_s >= len(done_before["S"]) - 1 and n_h >= len(done_before["H"])
+
+
+def _pair_events(m, tiles):
+    """The epilogue warps' hand-over events of a CTA with `tiles` tiles at d_model 128, in
+    program order (two tiles in turn, a last one by itself), restated from their loop:
+    (event, tile of the pair) with the events of _epilogue_events."""
+    NDC, L = m.d_hidden // 64, m.n_layers
+    ev = [("S", u) for u in range(min(tiles, 2))]         # the first tiles' Fourier operands
+    for j in range(0, tiles, 2):
+        us = range(2 if j + 1 < tiles else 1)
+        for u in us:
+            ev += [("W", u), ("S", u)]                    # embedding product 1 -> its SiLU
+        for u in us:
+            ev += [("W", u), ("S", u)]                    # embedding product 2 -> x_hat
+        for l in range(L):
+            for dc in range(NDC):
+                for u in us:
+                    ev += [("W", u), ("S", u)] + ([("B", u)] if dc > 0 else []) + [("H", u)]
+            for _ in ("gate", "mlp1"):
+                for u in us:
+                    ev += [("W", u), ("S", u)]
+            for u in us:                                  # MLP2 -> x_hat, or the next pair's operand
+                ev += [("W", u)] + ([("S", u)] if l + 1 < L or j + 2 + u < tiles else [])
+    return ev
+
+
+def _pair_issue(m, tiles):
+    """The issuer's events of the same CTA: ("S" | "H", tile) hand-overs consumed, ("W" | "B",
+    tile) commits made."""
+    one = T.schedule_counts(m, with_codes=True)["codes"]
+    two = T.schedule_counts(m, with_codes=True, two=True)["codes"]
+    out = []
+    for j in range(0, tiles, 2):
+        for c in two if j + 1 < tiles else [(c & 3) | (c >> 2) << 3 for c in one]:
+            u, wait, commit = c >> 5, c & 7, (c >> 3) & 3
+            out += [("S", u)] * (wait & 1) + [("S", u ^ 1)] * (wait >> 2) + [("H", u)] * ((wait >> 1) & 1)
+            out += [("W", u)] if commit == 1 else [("B", u)] if commit == 2 else []
+    return out
+
+
+@pytest.mark.parametrize("L", [1, 2, 6, 16])
+@pytest.mark.parametrize("tiles", [1, 2, 3, 4, 5])
+def test_two_tiles_in_turn_hand_over_soundly(lib, L, tiles):
+    """Two tiles in turn: each commit has its wait and each hand-over its consumer, nothing
+    stalls, and the barriers suffice whatever the warps' speeds.  Per tile the operand
+    hand-overs and the accumulator commits alternate between two barriers (a warp may be one
+    ahead, but give hand-over k + 2 only after all gave k; commit k + 2 may come only after
+    every warp has left its wait for k), the state ones use one (one less of each)."""
+    m = W.ModelConfig(max_hits=24, d_model=128, d_hidden=192, n_layers=L, precision=W.PRECISION_BF16)
+    epi, iss = _pair_events(m, tiles), _pair_issue(m, tiles)
+    for e in "SHWB":
+        for u in (0, 1):
+            assert epi.count((e, u)) == iss.count((e, u)), (e, u)
+    # both sides in program order, each waiting for the other: they reach their ends
+    given, made, i, k = {}, {}, 0, 0
+    taken, waited = {}, {}
+    while i < len(epi) or k < len(iss):
+        at = (i, k)
+        while i < len(epi) and (epi[i][0] in "SH" or waited.get(epi[i], 0) < made.get(epi[i], 0)):
+            t = given if epi[i][0] in "SH" else waited
+            t[epi[i]] = t.get(epi[i], 0) + 1
+            i += 1
+        while k < len(iss) and (iss[k][0] in "WB" or taken.get(iss[k], 0) < given.get(iss[k], 0)):
+            t = made if iss[k][0] in "WB" else taken
+            t[iss[k]] = t.get(iss[k], 0) + 1
+            k += 1
+        assert (i, k) != at, f"stalled at epilogue {epi[i:i + 1]}, issuer {iss[k:k + 1]}"
+    # hand-overs consumed before each commit, and waits left before each hand-over
+    n, before_commit = {}, {}
+    for e in iss:
+        if e[0] in "SH":
+            n[e] = n.get(e, 0) + 1
+        else:
+            before_commit.setdefault(e, []).append(dict(n))
+    seen, count, n, before_hand = {}, {}, {}, {}
+    for e in epi:
+        if e[0] in "WB":
+            for x, v in before_commit[e][count.get(e, 0)].items():
+                seen[x] = max(seen.get(x, 0), v)          # every warp has given v of x by now
+            count[e] = count.get(e, 0) + 1
+            n[e] = n.get(e, 0) + 1
+        else:
+            s, ahead = count.get(e, 0), 1 if e[0] == "S" else 0
+            assert s - seen.get(e, 0) <= ahead, (e, s)
+            count[e] = s + 1
+            before_hand.setdefault(e, []).append(dict(n))
+    left, count = {}, {}
+    for e in iss:
+        if e[0] in "SH":
+            for x, v in before_hand[e][count.get(e, 0)].items():
+                left[x] = max(left.get(x, 0), v)          # every warp has left v waits for x by now
+        else:
+            c, behind = count.get(e, 0), 2 if e[0] == "W" else 1
+            assert c < behind or left.get(e, 0) >= c - behind + 1, (e, c)
+        count[e] = count.get(e, 0) + 1
+
+
+def test_two_tiles_in_turn_do_two_tiles_work(lib):
+    m = W.ModelConfig(max_hits=24, d_model=128, d_hidden=192, n_layers=3, precision=W.PRECISION_FP16)
+    one, two = T.schedule_counts(m), T.schedule_counts(m, two=True)
+    assert two == {k: 2 * v for k, v in one.items()}
+    wide = m.with_(d_model=256, d_hidden=384)
+    assert set(T.schedule_counts(wide, two=True).values()) == {0}
