@@ -41,7 +41,7 @@ from paper_2609_32479_gb300 import workloads as W  # noqa: E402
 METRIC = "tracks/sec at 1 GB300 (device-timed) and % of HBM/tensor roofline vs CPU oracle"
 FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}
 KERNEL_SRC = tuple(os.path.join(ROOT, "paper_2609_32479_gb300", "csrc", f)
-                   for f in ("tc_forward.cu", "tc_epilogue.cuh"))
+                   for f in ("tc_forward.cu", "tc_epilogue.cuh", "sm100_ptx.cuh"))
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "tc_forward_large.traffic.json")
 
 
@@ -537,6 +537,18 @@ def code_digest(paths) -> str:
     return hashlib.sha256(" ".join(src.split()).encode()).hexdigest()
 
 
+def kernel_name(path, m) -> str:
+    """The kernel behind the library's timing hook for this path and model."""
+    if path.startswith("tcgen05-rows"):
+        return "concat_kernel" if m.topology == W.TOPOLOGY_CONCAT else "transformer_kernel"
+    if path.startswith("tcgen05"):
+        return "tc_pair_kernel" if m.d_model == 128 else "tc_forward_kernel"
+    # the fused fp32 encoder's rows fit shared memory up to these widths
+    if m.precision == W.PRECISION_FP32 and m.topology == W.TOPOLOGY_MERGE and m.d_model <= 128 and m.n_features <= 12:
+        return "encoder_fp32_kernel"
+    return "CUDA-core encoder, a launch a step"
+
+
 def traffic_for_kernel():
     """dram bytes per launch from the committed ncu summary, if it was taken on the
     current kernel code (else null)."""
@@ -701,8 +713,7 @@ def main():
                 "frac": (achieved / peak) if achieved else None, "traffic": traffic,
                 "peak_kind": peak_kind,
                 "frac_of_sustained": (achieved / peak_sus) if achieved else None,
-                "kernel": ("tc_pair_kernel" if m.d_model == 128 else "tc_forward_kernel") if tf.path.startswith("tcgen05")
-                          else "encoder_fp32_kernel",
+                "kernel": kernel_name(tf.path, m),
                 "kernel_ms_avg": kern_avg_s * 1e3, "launches_per_step": launches_per_step,
                 "flops_per_launch": flops_launch,
                 "algorithmic_bytes_per_launch": B * bytes_per_track(m) / launches_per_step,

@@ -50,3 +50,20 @@ def test_oracle_pool_matches_one_process():
     assert pool.workers >= 1
     assert got.shape == ref.shape
     np.testing.assert_allclose(got, ref, rtol=1e-11, atol=1e-13)
+
+
+def test_kernel_names():
+    """What the bench line calls the timed kernel: the fused fp32 encoder only for the models
+    that it takes, and the profile's digest covers every source of the wide kernel."""
+    sys.path.insert(0, ROOT)
+    import bench
+    from paper_2609_32479_gb300 import workloads as W
+    tiny, large = W.workload("tiny").model, W.workload("large").model
+    assert bench.kernel_name("simt-fp32", tiny) == "encoder_fp32_kernel"
+    for m, path in ((tiny.with_(precision=W.PRECISION_BF16), "simt-bf16"), (large.with_(precision=W.PRECISION_FP32), "simt-fp32"),
+                    (W.workload("paper").model.with_(precision=W.PRECISION_FP32), "simt-fp32")):
+        assert bench.kernel_name(path, m) == "CUDA-core encoder, a launch a step"
+    assert bench.kernel_name("tcgen05-bf16", W.workload("medium").model) == "tc_pair_kernel"
+    assert bench.kernel_name("tcgen05-bf16", large) == "tc_forward_kernel"
+    assert bench.kernel_name("tcgen05-rows-fp16", W.workload("paper").model) == "concat_kernel"
+    assert {os.path.basename(f) for f in bench.KERNEL_SRC} == {"tc_forward.cu", "tc_epilogue.cuh", "sm100_ptx.cuh"}
