@@ -21,7 +21,7 @@
 // concatenation topology) and the attention within each track (the Transformer),
 // the pooling and the head.
 //
-// Kernel roles (192 threads, one CTA per SM, persistent over 128-row x Nt tiles):
+// Kernel roles (320 threads, one CTA per SM, persistent over 128-row x Nt tiles):
 //   warp 0     TMA producer (one elected lane): A and W chunks of 64 k into a ring of stages
 //   warp 1     MMA issuer (one elected lane) and TMEM owner: two accumulator buffers
 //   warps 2-9  epilogue, TMEM lane quadrant = warp % 4, column half = (warp - 2) / 4
