@@ -194,12 +194,11 @@ __device__ void perigee_from_triplet(const double (&a)[3], const double (&b)[3],
 //
 // The fp64 pipe bounds this.  So the angle is evaluated once: the sine and cosine of
 // the direction at the start are the hit's own unit vector from the centre, and each
-// step turns them by the small angle of the step.  g'' is sin^2(theta) times the distance w
-// of the hit from the foot point along the transverse direction, so the angle is off by at
-// most d^2 w / 2 |g'| after a step d: one of 1e-5 is the last if w is below |g'| / 500 (g' is
-// near R / sin(theta): hits within a millimetre or so; it leaves 1e-13), else one of 1e-8.
-// (With 1e-5 for every hit s was up to 5e-9 off for hits 100 mm beside the helix, 2e-8 at
-// 1 m, near fp32's rounding.)
+// step turns them by the small angle of the step.  With w the distance of the hit from the
+// foot point along the transverse direction, g'' is sin^2(theta) w and g''' at most about
+// R / sin(theta), so after a step d the angle is off by less than d^2 (w + d R / sin(theta)) /
+// 2 |g'|: a step that leaves 1e-14 is the last.  (With a step of 1e-5 as the last s was up to
+// 5e-9 off for hits 100 mm beside the helix, 2e-8 at 1 m, near fp32's rounding.)
 __device__ __forceinline__ void residuals(const Helix& h, double x, double y, double z, double& du, double& dv,
                                           double& s) {
   double hx = x - h.cx, hy = y - h.cy;
@@ -228,7 +227,8 @@ __device__ __forceinline__ void residuals(const Helix& h, double x, double y, do
     const double s1 = sphi * cd + cphi * sd;
     cphi = cphi * cd - sphi * sd;
     sphi = s1;
-    if (fabs(d) <= (500.0 * fabs(w) <= fabs(dg) ? 1e-5 : 1e-8)) it = NEWTON_MAX - 1;   // one more pass for the residual, then out
+    // one more pass for the residual, then out
+    if (d * d * fma(fabs(d), h.r_st, fabs(w)) <= 2e-14 * fabs(dg)) it = NEWTON_MAX - 1;
   }
   // U = (-sin phi, cos phi, 0); V = t x U = (-cos theta cos phi, -cos theta sin phi, sin theta)
   du = ry * cphi - rx * sphi;
