@@ -208,7 +208,7 @@ def test_packing_segments_do_not_matter_to_a_track(T, n, hits):
 
 
 def test_hit_rows_of_fifteen_features_in_host_buffers_and_chunks(T):
-    """Hit rows wider than five features: from host buffers (copied whole, in two steps),
+    """Hit rows wider than five features: from host buffers (copied whole; in two steps below),
     and on the CUDA cores past the workspace's first chunk of tracks (4,923 of these)."""
     w = W.workload("paper", n_tracks=33000)
     tb = W.gen_tracks(w)
