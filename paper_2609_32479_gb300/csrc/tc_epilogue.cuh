@@ -518,7 +518,8 @@ __device__ __forceinline__ void scan_chain(const ECtx& x, float (&a)[32], const 
 // needs a finite state before it, or an infinity or NaN of one track would reach the next
 // in its slab.  So a column whose residual stream is not finite has x_hat 0 (ep_residual) and
 // with it finite gates and candidates; the stream itself keeps the column's value, adds to
-// it and is pooled, so the track's own result is no number either way.  Selecting at
+// it and is pooled, so the track's own result is no number either way.  (x_hat itself is at
+// most sqrt(d_model) times the gain, within 16 bits for any gain below 4,000.)  Selecting at
 // every restart instead cost 12 % (262,144 tracks of six layers, 12.1 to 13.5 ms).
 template <bool FP16>
 __device__ __forceinline__ void scan_chain_store(const ECtx& x, float (&a)[32], const float (&b)[32]) {
